@@ -1,7 +1,7 @@
 // Sparse gated FFN for one decode token per sequence (Algorithm 2, generation phase):
 //   kept = { j : A_j >= tau_final },  y = sum_{j in kept} silu(w_gate_j . x) (w_up_j . x) w_down_t[j,:]
 //
-// One persistent cooperative kernel per (layer, sequence), one CTA per SM:
+// One persistent kernel per (layer, sequence), one CTA per SM:
 //   prologue  every CTA tests all F scores against tau (the vector arrives as one bulk copy into the idle
 //             ring; a warp tests 32 chunks of 32 neurons with one ballot each), a block scan ranks the
 //             chunks, and the CTA takes an equal share [r0, r1) of the kept neurons in ascending order,
@@ -12,8 +12,8 @@
 //             thread t owns the same 16-byte column vectors of every row (x and the partial y for
 //             those columns live in registers) and reads the staged rows from shared memory, four
 //             neurons per CTA-wide reduction;
-//   epilogue  each CTA stores its fp32 partial y, all CTAs meet at a bounded grid barrier, then every
-//             CTA sums a slice of columns over all partials in CTA order (deterministic) and writes y.
+//   epilogue  each CTA stores its fp32 partial y, the CTAs meet (grid_meet), then every CTA sums a slice of
+//             columns over all partials in CTA order (deterministic) and writes y.
 #include <math.h>
 
 #include "common.cuh"
@@ -69,7 +69,10 @@ sparse_ffn_kernel(const FfnParams p, const int n_stages) {
         mbar_init(sbar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    __shared__ int s_all;  // every CTA of the launch has begun
+    if (tid == 0) s_all = 0;
     pdl_wait();  // everything below may read what the previous kernel wrote
+    if (tid == 0) grid_enter(p.ctrl);
 
     const uint64_t keep_policy = policy_evict_last();
     const bool nested = p.order != nullptr;
@@ -245,7 +248,7 @@ sparse_ffn_kernel(const FfnParams p, const int n_stages) {
     const int my_n = r1 - r0;
     if (n_act == 0) {
         // Nothing is kept (every CTA sees the same count): y = 0, written slice by slice, and there are
-        // no partial sums to combine, so the grid barrier is skipped as well.
+        // no partial sums to combine, so the meeting is skipped as well.
         const int ng = d / 4;  // output in groups of 4 columns
         const int q0 = split_at(ng, cta, n_ctas), q1 = split_at(ng, cta + 1, n_ctas);
         for (int q = q0 + tid; q < q1; q += kFfnThreads) {
@@ -254,6 +257,7 @@ sparse_ffn_kernel(const FfnParams p, const int n_stages) {
             else
                 reinterpret_cast<uint2 *>(p.y)[q] = make_uint2(0u, 0u);
         }
+        if (tid == 0) grid_leave(p.ctrl, (unsigned)n_ctas);
         return;
     }
     __syncthreads();  // s_list and the mbarriers are ready
@@ -287,6 +291,7 @@ sparse_ffn_kernel(const FfnParams p, const int n_stages) {
                     par ^= 1;
                 }
             }
+            if (grid_all_started(p.ctrl, (unsigned)n_ctas)) s_all = 1;
             // Never leave with copies in flight: the last use of every stage must have landed.
             for (int i = max(0, issued - n_stages); i < issued; ++i)
                 if (!mbar_wait(full0 + 8 * (i % n_stages), (i / n_stages) & 1)) timed_out = true;
@@ -315,17 +320,17 @@ sparse_ffn_kernel(const FfnParams p, const int n_stages) {
     }
     if (timed_out && p.status) atomicOr(p.status, CLADA_STATUS_TIMEOUT);
 
-    // ---- epilogue: grid barrier, deterministic column reduction ---------------------------------
-    if (!grid_barrier(p.ctrl, (unsigned)n_ctas, kConsumers)) {
-        if (tid == 0 && p.status) atomicOr(p.status, CLADA_STATUS_TIMEOUT);
-        return;
-    }
+    // ---- epilogue: the CTAs meet, deterministic column reduction --------------------------------
+    const GridMeet how = grid_meet(p.ctrl, (unsigned)n_ctas, kConsumers, &s_all);
+    if (how == kMeetTimeout && tid == 0 && p.status) atomicOr(p.status, CLADA_STATUS_TIMEOUT);
+    if (how == kMeetTimeout || how == kMeetLeave) return;
+    const int q_first = how == kMeetWhole ? warp : cta + warp * n_ctas, q_step = how == kMeetWhole ? kFfnWarps : n_ctas * kFfnWarps;
     // columns in groups of 4 (float4); a warp sums one group: lane l adds partial rows l, l+32, ... (one row
     // per CTA and consumer group) in order (five loads in flight at a time), then the 32 lane sums combine by
     // butterfly.
     const int ngroups = d / 4;
     const int n_rows = n_ctas * GROUPS;
-    for (int q = cta + warp * n_ctas; q < ngroups; q += n_ctas * kFfnWarps) {
+    for (int q = q_first; q < ngroups; q += q_step) {
         float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
         for (int rb = 0; rb < n_rows; rb += 5 * kWarp) {
             float4 v[5];
@@ -381,13 +386,11 @@ static int launch_variant(const FfnParams &p, cudaStream_t st) {
     cfg.blockDim = dim3(kFfnThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeCooperative;  // all CTAs co-resident: the grid barrier cannot starve
-    attr[0].val.cooperative = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // hide the launch latency
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // hide the launch latency
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 2;
+    cfg.numAttrs = 1;
     CLADA_CUDA_TRY(cudaLaunchKernelExC(&cfg, reinterpret_cast<const void *>(kern), args));
     return CLADA_OK;
 }

@@ -55,7 +55,10 @@ sparse_ffn_batch_kernel(const FfnBatchParams p, const int n_stages) {
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    __shared__ int s_all;  // every CTA of the launch has begun
+    if (tid == 0) s_all = 0;
     pdl_wait();
+    if (tid == 0) grid_enter(p.ctrl);
 
     const uint64_t keep_policy = policy_evict_last();
     if (tid < BT) s_tau[tid] = ld_keep(p.tau + (size_t)tid * p.tau_stride, keep_policy);
@@ -106,6 +109,7 @@ sparse_ffn_batch_kernel(const FfnBatchParams p, const int n_stages) {
                     par ^= 1;
                 }
             }
+            if (grid_all_started(p.ctrl, (unsigned)n_ctas)) s_all = 1;
             for (int i = max(0, issued - n_stages); i < issued; ++i)
                 if (!mbar_wait(full0 + 8 * (i % n_stages), (i / n_stages) & 1)) timed_out = true;
         }
@@ -248,12 +252,11 @@ sparse_ffn_batch_kernel(const FfnBatchParams p, const int n_stages) {
     }
     if (timed_out && p.status) atomicOr(p.status, CLADA_STATUS_TIMEOUT);
 
-    // ---- epilogue: grid barrier, deterministic column reduction per sequence ----------------------
-    if (!grid_barrier(p.ctrl, (unsigned)n_ctas, kConsumers)) {
-        if (tid == 0 && p.status) atomicOr(p.status, CLADA_STATUS_TIMEOUT);
-        return;
-    }
-    batch_column_sums<BT>(p);
+    // ---- epilogue: the CTAs meet, deterministic column reduction per sequence --------------------
+    const GridMeet how = grid_meet(p.ctrl, (unsigned)n_ctas, kConsumers, &s_all);
+    if (how == kMeetTimeout && tid == 0 && p.status) atomicOr(p.status, CLADA_STATUS_TIMEOUT);
+    if (how == kMeetTimeout || how == kMeetLeave) return;
+    batch_column_sums<BT>(p, how == kMeetWhole);
 }
 
 
@@ -340,13 +343,11 @@ static int launch_batch_variant(const FfnBatchParams &p, cudaStream_t st) {
     cfg.blockDim = dim3(kFfnThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeCooperative;  // all CTAs co-resident: the grid barrier cannot starve
-    attr[0].val.cooperative = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 2;
+    cfg.numAttrs = 1;
     CLADA_CUDA_TRY(cudaLaunchKernelExC(&cfg, reinterpret_cast<const void *>(kern), args));
     return CLADA_OK;
 }

@@ -29,13 +29,13 @@
 // Asking phase 2's boxes into L2 meanwhile (cp.async.bulk.prefetch.tensor, 8 to 48 stages) cost
 // 2.5 to 8 us: the requests are paid for twice.
 //
-// Work split: 4 consecutive CTAs form a group.  Member m of group g streams the gate / up rows of its own
+// Work split: 4 CTAs that begin one after another form a group.  Member m of group g streams the gate / up rows of its own
 // rows_blk neurons (phase 1), the four members exchange their parts of h through global memory (each writes its
 // slice of the operand image, a byte counter per group in the control block, bounded wait; the producer keeps
 // prefetching meanwhile), and in phase 2 member m streams column slice m (a quarter of d_model) of the down rows
 // of all four members' neurons, column tile by column tile, so that a finished tile's partial output is stored
 // while the next tile streams.  Every weight byte is read once, and a group writes ONE partial output
-// [B, d_model] instead of one per CTA.  After a grid barrier all threads sum the groups' partials in group order
+// [B, d_model] instead of one per CTA.  After the CTAs have met (grid_meet) all threads sum the groups' partials in group order
 // and write y.
 //
 // One persistent CTA per SM, 320 threads: warp 0 TMA producer (64-column boxes of rows_blk rows, 128-byte swizzle,
@@ -67,6 +67,7 @@ __host__ __device__ constexpr uint32_t bd_img_block(int seqs) { return (uint32_t
 constexpr int bd_tiles_in_tmem(int seqs) { return (int)kBdTmemCols / (kBdParts * seqs); }
 constexpr int kBdGroupWord0 = 8;     // group byte counters: control-block words 8..63
 constexpr int kBdMaxGroups = 4 * (64 - kBdGroupWord0);
+constexpr size_t kBdSmemMin = 120 * 1024;
 constexpr unsigned kBdGroupSpinLimit = 1u << 22;
 
 // Opt-in timeline (-DCLADA_BD_TRACE): %globaltimer stamps per CTA, 64 slots, written by the thread that passes the point.
@@ -192,13 +193,10 @@ sparse_ffn_batch_dense_kernel(const __grid_constant__ CUtensorMap map_x, const _
     __shared__ __align__(8) uint64_t s_full[kBdMaxStages], s_empty[kBdMaxStages], s_p1_full, s_h_own, s_h_all,
         s_tile_full[kBdMaxTiles], s_tile_read[kBdMaxTiles];
     __shared__ uint32_t s_tmem_base;
-    __shared__ int s_abort, s_group_ok;
+    __shared__ int s_abort, s_group_ok, s_cta, s_all;
 
     constexpr int kPer = SEQS / 2;  // sequences of an epilogue warp
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int cta = blockIdx.x;
-    const int grp = cta / kBdMembers, mem = cta - grp * kBdMembers;
-    const bool active = grp < p.n_groups;  // the CTAs behind the last whole group only join the barrier and the sums
     const bool gated = act_is_gated(p.act);
     const int n_kblocks = (p.d_model + kTcTileK - 1) / kTcTileK;
     const int n_stages = p.n_stages;
@@ -208,9 +206,6 @@ sparse_ffn_batch_dense_kernel(const __grid_constant__ CUtensorMap map_x, const _
     const int kimg_blocks = (kBdMembers * p.rpad + 63) / 64;
     const uint32_t img_bytes = (uint32_t)kimg_blocks * bd_img_block(SEQS);
     const uint32_t himg_s = smem0 + (uint32_t)n_stages * stage_bytes;  // the group's h image in shared memory
-    const int t0 = mem * p.tps;
-    const int nt = max(0, min(p.tps, p.n_tiles - t0));          // this member's column tiles in phase 2
-    const int j0 = cta * p.rows_blk;                            // this CTA's first neuron
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < n_stages; ++s) {
@@ -226,6 +221,7 @@ sparse_ffn_batch_dense_kernel(const __grid_constant__ CUtensorMap map_x, const _
         }
         s_abort = 0;
         s_group_ok = 0;
+        s_all = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     // Rows rows_blk .. rpad-1 of every box slot are never written by a copy but are read by the last K step of
@@ -253,6 +249,17 @@ sparse_ffn_batch_dense_kernel(const __grid_constant__ CUtensorMap map_x, const _
     volatile int *abort_flag = &s_abort;
     pdl_launch_dependents();
     pdl_wait();  // x, the scores and the thresholds may come from the launch before
+    // CTAs are numbered in the order in which they begin.  The launch is a plain one, so nothing promises that all CTAs
+    // are resident at a time; but with these numbers every group but the last one begun is complete whenever a CTA
+    // waits, goes through to the end by itself and makes room for the others.
+    if (threadIdx.x == 0) s_cta = (int)grid_enter(p.ctrl);
+    __syncthreads();
+    const int cta = s_cta;
+    const int grp = cta / kBdMembers, mem = cta - grp * kBdMembers;
+    const bool active = grp < p.n_groups;  // the CTAs behind the last whole group only join the meeting and the sums
+    const int t0 = mem * p.tps;
+    const int nt = max(0, min(p.tps, p.n_tiles - t0));          // this member's column tiles in phase 2
+    const int j0 = cta * p.rows_blk;                            // this CTA's first neuron
     if (threadIdx.x == 0) BD_TRACE(0);
 
     if (active && warp == 0) {
@@ -304,6 +311,7 @@ sparse_ffn_batch_dense_kernel(const __grid_constant__ CUtensorMap map_x, const _
             }
             BD_TRACE(15);
             if (!ok) *abort_flag = 1;
+            if (grid_all_started(p.ctrl, gridDim.x)) s_all = 1;
             for (int i = max(0, kc - n_stages); i < kc; ++i) {  // never leave with copies in flight
                 int never = 0;
                 if (!tc_mbar_wait(tc_smem_u32(&s_full[i % n_stages]), (i / n_stages) & 1, &never)) *abort_flag = 1;
@@ -559,18 +567,19 @@ sparse_ffn_batch_dense_kernel(const __grid_constant__ CUtensorMap map_x, const _
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kBdTmemCols) : "memory");
     }
-    // ---- all groups' partial outputs are in global memory after the barrier: sum them in group order ----------
-    if (!grid_barrier(p.ctrl, gridDim.x, 32)) {
-        if (threadIdx.x == 0 && p.status) atomicOr(p.status, CLADA_STATUS_TIMEOUT);
-        return;
-    }
+    // ---- all groups' partial outputs are in global memory after the meeting: sum them in group order ----------
+    const GridMeet how = grid_meet(p.ctrl, gridDim.x, 32, &s_all);
+    if (how == kMeetTimeout && threadIdx.x == 0 && p.status) atomicOr(p.status, CLADA_STATUS_TIMEOUT);
+    if (how == kMeetTimeout || how == kMeetLeave) return;
     if (threadIdx.x == 0) BD_TRACE(12);
-    if (cta == 0 && threadIdx.x < 64 - kBdGroupWord0)  // every member has passed its group's counter: clear them
+    const bool whole = how == kMeetWhole;
+    if ((cta == 0 || whole) && threadIdx.x < 64 - kBdGroupWord0)  // every member has passed its group's counter: clear them
         reinterpret_cast<unsigned *>(p.ctrl)[kBdGroupWord0 + threadIdx.x] = 0u;
     const int d4 = p.d_model / 4;
-    const int share = (p.B * d4 + gridDim.x - 1) / gridDim.x;  // every CTA takes an equal run of (sequence, four columns)
-    const int it1 = min(p.B * d4, (cta + 1) * share);
-    for (int it = cta * share + threadIdx.x; it < it1; it += kBdThreads) {
+    // every CTA takes an equal run of (sequence, four columns)
+    const int share = whole ? p.B * d4 : (p.B * d4 + gridDim.x - 1) / gridDim.x;
+    const int it0 = whole ? 0 : cta * share, it1 = min(p.B * d4, it0 + share);
+    for (int it = it0 + threadIdx.x; it < it1; it += kBdThreads) {
         const int b = it / d4, q = it - b * d4;
         float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
         const float4 *src = reinterpret_cast<const float4 *>(p.partials) + (size_t)b * d4 + q;
@@ -628,7 +637,9 @@ static bool bd_plan(const clada_layer *layer, int B, const DeviceInfo &di, BdPla
     const size_t tail = std::max<size_t>(pl->himg_bytes, 16384);
     if (budget < 1024 + tail + 3 * stage_bytes) return false;
     pl->n_stages = (int)std::min<size_t>(kBdMaxStages, (budget - 1024 - tail) / stage_bytes);
-    pl->smem = 1024 + (size_t)pl->n_stages * stage_bytes + tail;
+    // never two CTAs on an SM (more than half of its shared memory): the second would wait for tensor memory that the
+    // first gives back only at its end
+    pl->smem = std::max<size_t>(1024 + (size_t)pl->n_stages * stage_bytes + tail, kBdSmemMin);
     pl->partial_bytes = (size_t)pl->n_groups * B * layer->d_model * sizeof(float);
     return true;
 }
@@ -706,13 +717,11 @@ int launch_ffn_batch_dense(const clada_layer *layer, int B, const void *x, const
     cfg.blockDim = dim3(kBdThreads);
     cfg.dynamicSmemBytes = pl.smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeCooperative;  // all CTAs co-resident: the group waits and the grid barrier cannot starve
-    attr[0].val.cooperative = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 2;
+    cfg.numAttrs = 1;
     CLADA_CUDA_TRY(cudaLaunchKernelExC(&cfg, kernel, args));
     return CLADA_OK;
 }

@@ -126,7 +126,10 @@ sparse_ffn_batch_tc_kernel(const FfnBatchParams p, const int n_slots) {
         for (int s = 0; s < n_slots; ++s) mbar_init(full0 + 8 * s, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    __shared__ int s_all;  // every CTA of the launch has begun
+    if (tid == 0) s_all = 0;
     pdl_wait();
+    if (tid == 0) grid_enter(p.ctrl);
     TC_TRACE(255, 0);
 
     const uint64_t keep_policy = policy_evict_last();
@@ -305,6 +308,7 @@ sparse_ffn_batch_tc_kernel(const FfnBatchParams p, const int n_slots) {
         TC_TRACE(g0 / CH, 6);
     }
     TC_TRACE(255, 3);
+    if (tid == kWarp && grid_all_started(p.ctrl, (unsigned)n_ctas)) s_all = 1;
     // Never leave with copies in flight.  Every copy issued was waited for above, unless a wait gave up: then
     // thread 0 waits (bounded again) for the last slots' worth.
     if (timed_out && tid == 0) {
@@ -326,13 +330,12 @@ sparse_ffn_batch_tc_kernel(const FfnBatchParams p, const int n_slots) {
     if (timed_out && p.status) atomicOr(p.status, CLADA_STATUS_TIMEOUT);
     TC_TRACE(255, 4);
 
-    // ---- epilogue: grid barrier, deterministic column reduction per sequence ----------------------
-    if (!grid_barrier(p.ctrl, (unsigned)n_ctas, kWarp)) {
-        if (tid == 0 && p.status) atomicOr(p.status, CLADA_STATUS_TIMEOUT);
-        return;
-    }
+    // ---- epilogue: the CTAs meet, deterministic column reduction per sequence --------------------
+    const GridMeet how = grid_meet(p.ctrl, (unsigned)n_ctas, kWarp, &s_all);
+    if (how == kMeetTimeout && tid == 0 && p.status) atomicOr(p.status, CLADA_STATUS_TIMEOUT);
+    if (how == kMeetTimeout || how == kMeetLeave) return;
     TC_TRACE(255, 5);
-    batch_column_sums<BT, kConsumers>(p);
+    batch_column_sums<BT, kConsumers>(p, how == kMeetWhole);
     TC_TRACE(255, 6);
 }
 
@@ -373,13 +376,11 @@ static int launch_tc_variant(const FfnBatchParams &p, cudaStream_t st) {
     cfg.blockDim = dim3(kConsumers);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeCooperative;  // all CTAs co-resident: the grid barrier cannot starve
-    attr[0].val.cooperative = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 2;
+    cfg.numAttrs = 1;
     CLADA_CUDA_TRY(cudaLaunchKernelExC(&cfg, reinterpret_cast<const void *>(kern), args));
     return CLADA_OK;
 }

@@ -5,7 +5,7 @@
 //
 // A launch per layer pays, per layer, for what does not move weight bytes: the launch ramp, the score
 // test, the first rows' latency, the slowest CTA's tail, a grid barrier and the column sums.  Here the
-// weight stream never stops at a layer boundary.  One cooperative CTA per SM, as in the per-layer kernel:
+// weight stream never stops at a layer boundary.  One cooperative CTA per SM:
 //   scanner   one warp builds the kept lists: it tests a layer's scores against its threshold and writes
 //             this CTA's equal share of the kept neurons into one of four list buffers, up to four layers
 //             ahead of the layer being streamed, so the score test is never on anybody's path.

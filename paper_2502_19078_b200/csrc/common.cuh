@@ -42,7 +42,8 @@ int device_info(DeviceInfo *out);
 constexpr size_t kWsCtrlBytes = 256;
 struct WsCtrl {
     unsigned int arrive;  // grid barrier: CTAs that reached it
-    unsigned int depart;  // CTAs that left it; the last one resets both
+    unsigned int depart;  // CTAs that left it; the last one resets all of these
+    unsigned int started; // CTAs that have begun (grid_enter)
 };
 
 // ---- device helpers -----------------------------------------------------------------------

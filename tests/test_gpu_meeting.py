@@ -1,0 +1,95 @@
+"""Decode launches whose CTAs cannot all be resident at a time: beside a kernel that keeps half of the SMs for longer than
+a decode takes, and beside another decode on a second stream.  Every launch ends, its control words are back at zero and
+its outputs are the bits of an undisturbed run."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def clada():
+    from paper_2502_19078_b200 import binding, build
+    build.build()
+    binding.load()
+    return binding
+
+
+def _layer(clada, d, F, dtype):
+    g = torch.Generator(device="cuda").manual_seed(d + F)
+    mk = lambda *s: torch.randn(s, generator=g, device="cuda").mul_(0.05).to(dtype)
+    return clada.Layer(mk(F, d), mk(F, d), mk(F, d))
+
+
+class _Decode:
+    def __init__(self, clada, B, d, F, dtype, nested):
+        self.clada, self.layer, self.nested = clada, _layer(clada, d, F, dtype), nested
+        g = torch.Generator(device="cuda").manual_seed(B)
+        self.x = torch.randn(B, d, generator=g, device="cuda").to(dtype)
+        self.scores = torch.rand(B, F, generator=g, device="cuda") + 0.5
+        self.tau = torch.full((B,), 0.8, device="cuda")
+        self.order = torch.empty(B, F, dtype=torch.int32, device="cuda")
+        self.counts = torch.empty(B, 4, dtype=torch.int32, device="cuda")
+        clada.clada_nested_build(self.scores, self.tau, 0.25, 0.1, self.order, self.counts)
+        self.level = torch.zeros(B, dtype=torch.int32, device="cuda")
+        self.ws, self.status = clada.new_workspace(self.layer, B, 0), torch.zeros(1, dtype=torch.int32, device="cuda")
+
+    def run(self):
+        y = torch.full(self.x.shape, float("nan"), device="cuda")
+        if self.nested:
+            self.clada.clada_sparse_ffn_decode_nested(self.layer, self.x, self.order, self.counts, self.level, y, self.ws,
+                                                      None, self.status)
+        else:
+            self.clada.clada_sparse_ffn_decode(self.layer, self.x, self.scores, self.tau, 1, y, self.ws, status=self.status)
+        return y
+
+    def clean(self):
+        return int(self.status.item()) == 0 and int(self.ws[:256].view(torch.int32).abs().sum().item()) == 0
+
+
+FORMS = [(1, 1024, 2400, torch.bfloat16, False), (1, 512, 1376, torch.float32, False), (2, 1024, 2400, torch.bfloat16, False),
+         (2, 512, 1376, torch.float32, False), (4, 512, 1376, torch.float32, False), (6, 1024, 2400, torch.float16, False),
+         (20, 1024, 2400, torch.bfloat16, False), (1, 1024, 2400, torch.bfloat16, True), (5, 1024, 2400, torch.bfloat16, True)]
+
+
+@pytest.mark.parametrize("B,d,F,dtype,nested", FORMS)
+def test_beside_a_kernel_that_keeps_half_of_the_sms(clada, B, d, F, dtype, nested):
+    dec = _Decode(clada, B, d, F, dtype, nested)
+    want = dec.run()
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    other_layer = _layer(clada, 8192, 128 * (sms // 2), torch.bfloat16)  # one persistent CTA per 128 neurons of one token tile
+    norm = torch.empty(other_layer.d_ff, device="cuda")
+    clada.clada_down_norms(other_layer, norm)
+    other_layer.set_down_norm(norm)
+    X, ws = torch.randn(128, 8192, device="cuda").to(torch.bfloat16), clada.new_workspace(other_layer, 1, 128)
+    scores = torch.empty(1, other_layer.d_ff, device="cuda")
+    other = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    outs = []
+    for _ in range(20):
+        with torch.cuda.stream(other):
+            clada.clada_prefix_scores(other_layer, X, [0, 128], scores, ws)
+        outs += [dec.run(), dec.run()]
+        torch.cuda.synchronize()
+    assert dec.clean()
+    for y in outs:
+        assert torch.equal(y, want)
+
+
+@pytest.mark.parametrize("first", range(len(FORMS)))
+def test_two_streams(clada, first):
+    """Launches of two streams that share the SMs as they come."""
+    decs = [_Decode(clada, *FORMS[first]), _Decode(clada, *FORMS[(first + 2) % len(FORMS)])]
+    want = [d.run() for d in decs]
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    torch.cuda.synchronize()
+    outs = [[], []]
+    for _ in range(40):
+        for i in (0, 1):
+            with torch.cuda.stream(streams[i]):
+                outs[i].append(decs[i].run())
+    torch.cuda.synchronize()
+    for i in (0, 1):
+        assert decs[i].clean()
+        for y in outs[i]:
+            assert torch.equal(y, want[i])
