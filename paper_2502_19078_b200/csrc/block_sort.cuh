@@ -22,17 +22,18 @@ constexpr size_t kSortSmem = (size_t)kSortMaxN * 8 + (size_t)(kSortBuckets + 1) 
 // elements per piece: count, scan, scatter, and every element's rank is its piece's start plus the number of smaller
 // (key, index) pairs in the piece.  Five passes over the elements instead of the 105 of the bitonic network, which
 // remains for keys that crowd into a piece (many equal scores).  Only the pieces that hold ranks of [r0, r1) are
-// scattered and ranked, so CTAs that share a sequence repeat the counting alone.  Bound by latency, memory's first and
-// shared memory's afterwards: 8 sequences of 14336 neurons take 198 us with the network, 19.1 us (cold caches)
-// with every element scattered by each of four CTAs, 14.2 us this way with eight.  The order inside a piece's slots is arrival order; the
-// ranks do not depend on it.
+// scattered and ranked (a comparison of piece numbers in registers tells which), so CTAs that share a sequence repeat the
+// counting alone.  Bound by latency, memory's first and shared memory's afterwards.  The order inside a piece's slots is
+// arrival order; the ranks do not depend on it.  Measured: lists of 8 sequences of 14336 neurons take 194.5 us a call with
+// the network, 12.5 with every element's piece looked up and the counters scanned one by one (a warp's in four banks), 11.5
+// now; 32 of them 14.0 / 12.5, 16 of 16384 13.7 / 12.2.
 template <typename Load, typename KeyOf, typename Emit>
 __device__ void block_sort(int n, unsigned reg_lo, unsigned reg_hi, int r0, int r1, unsigned char *smem, Load load,
                            KeyOf key_of, Emit emit) {
     unsigned long long *s_key = reinterpret_cast<unsigned long long *>(smem);
     int *s_cnt = reinterpret_cast<int *>(smem + (size_t)kSortMaxN * 8);
     __shared__ unsigned s_min[kSortThreads / kWarp], s_max[kSortThreads / kWarp];
-    __shared__ int s_wtot[kSortThreads / kWarp], s_wmax[kSortThreads / kWarp], s_edge[2];
+    __shared__ int s_wtot[kSortThreads / kWarp], s_wmax[kSortThreads / kWarp], s_edge[2], s_piece[2];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
     unsigned key[kSortPer], slot[kSortPer];
@@ -80,10 +81,16 @@ __device__ void block_sort(int n, unsigned reg_lo, unsigned reg_hi, int r0, int 
     __syncthreads();
     // exclusive scan of the counters (eight consecutive ones per thread) and the fullest piece
     constexpr int kPer = kSortBuckets / kSortThreads;
+    static_assert(kPer % 4 == 0, "counters as 16-byte vectors (one by one a warp's would share four banks)");
+    int4 *own = reinterpret_cast<int4 *>(s_cnt + tid * kPer);
     int c[kPer], sum = 0, fullest = 0;
 #pragma unroll
+    for (int q = 0; q < kPer; q += 4) {
+        const int4 v = own[q / 4];
+        c[q] = v.x; c[q + 1] = v.y; c[q + 2] = v.z; c[q + 3] = v.w;
+    }
+#pragma unroll
     for (int q = 0; q < kPer; ++q) {
-        c[q] = s_cnt[tid * kPer + q];
         sum += c[q];
         fullest = max(fullest, c[q]);
     }
@@ -100,26 +107,35 @@ __device__ void block_sort(int n, unsigned reg_lo, unsigned reg_hi, int r0, int 
     fullest = __reduce_max_sync(0xffffffffu, s_wmax[lane]);
     if (fullest <= kSortMaxBucket) {
         int base = __reduce_add_sync(0xffffffffu, lane < warp ? s_wtot[lane] : 0) + incl - sum;
+        int start[kPer];
 #pragma unroll
         for (int q = 0; q < kPer; ++q) {
-            s_cnt[tid * kPer + q] = base;
+            start[q] = base;
             base += c[q];
+            // the pieces that hold the first and the last rank asked for
+            if (start[q] <= r0 && r0 < base) {
+                s_piece[0] = tid * kPer + q;
+                s_edge[0] = start[q];
+            }
+            if (start[q] < r1 && r1 <= base) {
+                s_piece[1] = tid * kPer + q;
+                s_edge[1] = base;
+            }
         }
+#pragma unroll
+        for (int q = 0; q < kPer; q += 4) own[q / 4] = make_int4(start[q], start[q + 1], start[q + 2], start[q + 3]);
         if (tid == kSortThreads - 1) s_cnt[kSortBuckets] = n;
         __syncthreads();
-        if (tid < 2) s_edge[tid] = tid == 0 ? n : 0;
-        __syncthreads();
-        // the positions of the pieces that hold ranks of [r0, r1)
+        if (r0 >= r1) return;
+        // scatter the elements of the pieces from one to the other
+        const int piece0 = s_piece[0], piece1 = s_piece[1];
 #pragma unroll
         for (int e = 0; e < kSortPer; ++e) {
             const int i = tid + e * kSortThreads;
             if (i < n) {
-                const int b = bucket_of(key[e]), first = s_cnt[b];
-                if (first < r1 && s_cnt[b + 1] > r0) {
-                    s_key[first + (int)slot[e]] = ((unsigned long long)key[e] << 32) | (unsigned)i;
-                    if (first <= r0) s_edge[0] = first;               // one piece only, whoever writes it
-                    if (s_cnt[b + 1] >= r1) s_edge[1] = s_cnt[b + 1];
-                }
+                const int b = bucket_of(key[e]);
+                if (b >= piece0 && b <= piece1)
+                    s_key[s_cnt[b] + (int)slot[e]] = ((unsigned long long)key[e] << 32) | (unsigned)i;
             }
         }
         __syncthreads();

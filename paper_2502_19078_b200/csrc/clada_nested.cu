@@ -112,7 +112,7 @@ nested_build_kernel(const float *__restrict__ scores, int d_ff, const float *__r
 // Layers of at most kSortMaxN neurons: one or a few CTAs per sequence sort in shared memory
 // (block_sort); each CTA of a sequence prepares the same table and writes its slice of the list, CTA 0 also counts.
 // Measured (lists of 8 sequences of 14336 neurons, back-to-back calls): 194.5 us a call with the bitonic network alone,
-// 16.4 us with four CTAs that each scatter everything, 12.7 now (13.2 with six CTAs, 14.0 with four).
+// 16.4 us with four CTAs that each scatter everything, 12.5 with eight (13.2 with six CTAs, 14.0 with four), 11.5 now.
 __global__ void __launch_bounds__(kSortThreads, 1)
 nested_sort_kernel(const float *__restrict__ scores, int d_ff, const float *__restrict__ tau_base,
                    long long tau_stride, const NestMults mults, int32_t *__restrict__ order,
