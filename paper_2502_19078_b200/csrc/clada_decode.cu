@@ -8,6 +8,7 @@
 #include "ffn_batch.cuh"
 #include "ffn_common.cuh"
 #include "ffn_single.cuh"
+#include "nested_batch.cuh"
 
 using namespace clada;
 
@@ -191,10 +192,11 @@ extern "C" int clada_sparse_ffn_decode(const clada_layer *layer, const void *x, 
 }
 
 // Decode from nested index lists (clada_nested_build): no scores, no threshold, no compaction -- the
-// kept set of sequence b is the leading counts[b][level[b]] entries of order[b].  One launch per sequence: only the
-// rows its own list names are read, and h stays in fp32.  (With a dense pass over the layer for three or more sequences
-// a step of four took 53 us instead of 100, 2048 x 16384 at 50 % kept; but an infinity in a row that nobody keeps, or an
-// fp16 layer's h beyond 65504, made every output NaN, and its sums are the tensor cores' truncated ones.)
+// kept set of sequence b is the leading counts[b][level[b]] entries of order[b].  Three to eight sequences at a time share
+// their reads (clada_nested_batch.cu) where the workspace holds such a pass, the others have a launch each; a sequence gets
+// the same bits either way: only rows that some list names are read, and h stays in fp32.  (The dense pass over the layer is
+// not for lists: an infinity in a row that nobody keeps, or an fp16 layer's h beyond 65504, made every output NaN, and its
+// sums are the tensor cores' truncated ones.)
 extern "C" int clada_sparse_ffn_decode_nested(const clada_layer *layer, const void *x, int32_t B,
                                               const int32_t *order, const int32_t *counts, const int32_t *level,
                                               void *y, int32_t y_dtype, int32_t *count_out, void *ws,
@@ -213,7 +215,20 @@ extern "C" int clada_sparse_ffn_decode_nested(const clada_layer *layer, const vo
     if (ws_bytes < decode_scratch_bytes(layer, 1, di.num_sms, 1)) return CLADA_ERR_WORKSPACE;
     const size_t esz = elem_size(layer->dtype), ysz = elem_size(y_dtype);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    for (int b = 0; b < B; ++b) {
+    for (int b = 0; b < B;) {
+        int nb = std::min(B - b, kNestedBatchMax);  // the most whose pass the workspace holds
+        while (nb >= kNestedBatchMin && (!nested_batch_supported(layer, nb) ||
+                                         ws_bytes < kWsCtrlBytes + nested_batch_scratch_bytes(layer, nb, di.num_sms)))
+            --nb;
+        if (nb >= kNestedBatchMin) {
+            rc = launch_nested_batch(layer, nb, static_cast<const char *>(x) + (size_t)b * layer->d_model * esz,
+                                     order + (size_t)b * layer->d_ff, counts + (size_t)b * 4, level + b,
+                                     static_cast<char *>(y) + (size_t)b * layer->d_model * ysz, y_dtype,
+                                     count_out ? count_out + b : nullptr, ws, status, st);
+            if (rc != CLADA_OK) return rc;
+            b += nb;
+            continue;
+        }
         FfnParams p = {};
         p.w_gate = layer->w_gate;
         p.w_up = layer->w_up;
@@ -233,6 +248,7 @@ extern "C" int clada_sparse_ffn_decode_nested(const clada_layer *layer, const vo
         p.level = level + b;
         rc = launch_ffn_single(p, layer->dtype, st);
         if (rc != CLADA_OK) return rc;
+        ++b;
     }
     return CLADA_OK;
 }

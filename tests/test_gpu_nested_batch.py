@@ -1,0 +1,81 @@
+"""Nested decode of several sequences in shared passes: every sequence gets the bits of a launch of its own, at the edges
+of its tiles (rows of one vector, of one or two consumer groups, of two vectors per thread; layers smaller than the grid;
+empty, whole and one-neuron lists; passes of two to eight sequences and rests), with any workspace that was accepted."""
+import pytest
+import torch
+
+from tests._util import launches
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def clada():
+    from paper_2502_19078_b200 import binding, build
+    build.build()
+    binding.load()
+    return binding
+
+
+def _case(clada, B, d, F, dtype, act):
+    g = torch.Generator(device="cuda").manual_seed(1000 * B + d + F)
+    mk = lambda s, *shape: torch.randn(shape, generator=g, device="cuda").mul_(s).to(dtype)
+    layer = clada.Layer(mk(0.05, F, d), None if act == 2 else mk(0.05, F, d), mk(0.05, F, d), activation=act)
+    order = torch.stack([torch.randperm(F, generator=g, device="cuda") for _ in range(B)]).to(torch.int32)
+    counts = torch.randint(0, F + 1, (B, 4), generator=g, device="cuda").to(torch.int32)
+    counts[0] = F                                            # everything kept
+    counts[1] = 0                                            # nothing kept
+    if B > 2:
+        counts[2] = 1
+    level = (torch.arange(B, device="cuda") % 4).to(torch.int32)
+    return layer, order, counts, level, mk(1.0, B, d)
+
+
+def _run(clada, layer, order, counts, level, x, y_dtype, ws):
+    y = torch.full((x.shape[0], x.shape[1]), 7.0, device="cuda").to(y_dtype)
+    kept = torch.full((x.shape[0],), -1, dtype=torch.int32, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    clada.clada_sparse_ffn_decode_nested(layer, x, order, counts, level, y, ws, kept, status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    assert kept.tolist() == [int(counts[b, int(level[b])]) for b in range(x.shape[0])]
+    return y
+
+
+@pytest.mark.parametrize("B,d,F,dtype,act", [
+    (2, 8, 1, torch.bfloat16, 0), (3, 8, 31, torch.float16, 1), (8, 2048, 147, torch.bfloat16, 0),
+    (4, 2048, 149, torch.bfloat16, 1), (9, 2056, 500, torch.float16, 0), (5, 2056, 333, torch.bfloat16, 2),
+    (2, 1024, 13400, torch.bfloat16, 2), (7, 4096, 1000, torch.bfloat16, 0), (3, 4104, 700, torch.float16, 0),
+    (8, 5120, 450, torch.bfloat16, 0), (3, 8192, 300, torch.bfloat16, 0), (6, 8192, 300, torch.float16, 2),
+    (3, 512, 1376, torch.float32, 0), (4, 1024, 640, torch.float32, 2), (8, 1032, 640, torch.float32, 1),
+    (3, 4096, 200, torch.float32, 0), (10, 256, 40000, torch.bfloat16, 0),
+])
+def test_batch_bits_are_those_of_single_launches(clada, B, d, F, dtype, act):
+    layer, order, counts, level, x = _case(clada, B, d, F, dtype, act)
+    ws, one = clada.new_workspace(layer, B, 0), clada.new_workspace(layer, 1, 0)
+    y = _run(clada, layer, order, counts, level, x, torch.float32, ws)
+    for b in range(B):
+        s = slice(b, b + 1)
+        assert torch.equal(y[s], _run(clada, layer, order[s], counts[s], level[s], x[s], torch.float32, one)), b
+    assert torch.all(y[1] == 0)
+    assert torch.equal(y, _run(clada, layer, order, counts, level, x, torch.float32, one))  # the smallest accepted workspace
+    h = dtype if dtype != torch.float32 else torch.float16
+    assert torch.equal(y.to(h), _run(clada, layer, order, counts, level, x, h, ws))          # 16-bit outputs: one rounding
+
+
+def test_repeated_indices_count_as_often_as_they_are_listed(clada):
+    layer, order, counts, level, x = _case(clada, 3, 512, 300, torch.bfloat16, 0)
+    order[0, 10:20] = order[0, 5]
+    ws = clada.new_workspace(layer, 3, 0)
+    y = _run(clada, layer, order, counts, level, x, torch.float32, ws)
+    for b in range(3):
+        s = slice(b, b + 1)
+        assert torch.equal(y[s], _run(clada, layer, order[s], counts[s], level[s], x[s], torch.float32, ws))
+
+
+def test_launches_do_not_grow_with_the_batch(clada):
+    """Four launches whatever the batch, not one per sequence."""
+    layer, order, counts, level, x = _case(clada, 8, 512, 1000, torch.bfloat16, 0)
+    ws, y = clada.new_workspace(layer, 8, 0), torch.empty(8, 512, device="cuda")
+    names = [n for n, _ in launches(lambda: clada.clada_sparse_ffn_decode_nested(layer, x, order, counts, level, y, ws))]
+    assert len(names) == 4 and not any("sparse_ffn_kernel" in n for n in names), names
