@@ -313,16 +313,28 @@ prefix_finalize_kernel(const float *__restrict__ partials, const SeqTable tab, i
 }
 
 // Chunked prefill: the same tile sums added into a running sum of squares per (prompt, neuron) ...
+// Latency-bound: with one load after the other 7.1 us for the 16 tiles of 2000 tokens (14336 neurons); its launch, the
+// finishing one and the down projection's are chained to what runs before them.  A chunk of 256 tokens (4096 x 11008), three
+// calls, 109 us before and 102.6 now, of 2000 tokens (4096 x 14336) 609 / 604.
 __global__ void prefix_accumulate_kernel(const float *__restrict__ partials, const SeqTable tab, int tile, int d_ff,
                                          float *__restrict__ sumsq) {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     const int b = blockIdx.y;
-    if (j >= d_ff) return;
     int first = 0;
     for (int q = 0; q < b; ++q) first += tiles_of(tab.off[q + 1] - tab.off[q], tile);
     const int n = tiles_of(tab.off[b + 1] - tab.off[b], tile);
+    pdl_launch_dependents();
+    pdl_wait();
+    if (j >= d_ff) return;
     float s = sumsq[(size_t)b * d_ff + j];
-    for (int t = 0; t < n; ++t) s += partials[(size_t)(first + t) * d_ff + j];
+    for (int t0 = 0; t0 < n; t0 += 16) {  // sixteen loads in flight, added in tile order
+        float v[16];
+#pragma unroll
+        for (int u = 0; u < 16; ++u) v[u] = t0 + u < n ? partials[(size_t)(first + t0 + u) * d_ff + j] : 0.f;
+#pragma unroll
+        for (int u = 0; u < 16; ++u)
+            if (t0 + u < n) s += v[u];
+    }
     sumsq[(size_t)b * d_ff + j] = s;
 }
 
@@ -330,6 +342,8 @@ __global__ void prefix_accumulate_kernel(const float *__restrict__ partials, con
 __global__ void prefix_finish_kernel(const float *__restrict__ sumsq, int B, int d_ff,
                                      const float *__restrict__ w_down_norm, float *__restrict__ scores) {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    pdl_launch_dependents();
+    pdl_wait();
     if (i >= (size_t)B * d_ff) return;
     scores[i] = __fmul_rn(sqrtf(sumsq[i]), w_down_norm[i % d_ff]);
 }
@@ -956,10 +970,8 @@ int clada_prefix_accumulate(const clada_layer *layer, const void *X, const int64
         if (rc != CLADA_OK) return rc;
         tile = kTcTokenTile;
     }
-    dim3 agrid((layer->d_ff + 255) / 256, tab.B);
-    prefix_accumulate_kernel<<<agrid, 256, 0, st>>>(partials, tab, tile, layer->d_ff, sumsq);
-    CLADA_CUDA_TRY(cudaGetLastError());
-    return CLADA_OK;
+    return launch_chained(prefix_accumulate_kernel, dim3((layer->d_ff + 127) / 128, tab.B), 128, st, partials, tab, tile, layer->d_ff,
+                          sumsq);
 }
 
 int clada_prefix_finish(const clada_layer *layer, const float *sumsq, int32_t B, float *scores, void *stream) {
@@ -969,10 +981,8 @@ int clada_prefix_finish(const clada_layer *layer, const float *sumsq, int32_t B,
     if (!sumsq || !scores) return CLADA_ERR_NULL;
     if (B <= 0) return CLADA_ERR_SHAPE;
     const size_t n = (size_t)B * layer->d_ff;
-    prefix_finish_kernel<<<(unsigned)((n + 255) / 256), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        sumsq, B, layer->d_ff, layer->w_down_norm, scores);
-    CLADA_CUDA_TRY(cudaGetLastError());
-    return CLADA_OK;
+    return launch_chained(prefix_finish_kernel, dim3((unsigned)((n + 255) / 256)), 256, static_cast<cudaStream_t>(stream), sumsq, B,
+                          layer->d_ff, layer->w_down_norm, scores);
 }
 
 int clada_prefill_down(const clada_layer *layer, const void *w_down, const void *Z, int64_t T, void *Y,
