@@ -402,7 +402,8 @@ int clada_prefill_down(const clada_layer *layer, const void *w_down, const void 
  * clada_sparse_ffn_decode_nested, per decode step and layer: the sparse FFN over
  * order[b][0 .. counts[b][level[b]]).  Same x / y / workspace / status rules as
  * clada_sparse_ffn_decode (workspace of clada_workspace_bytes(layer, 1, 0) is
- * enough); sequences run one launch each.  The sum over the kept neurons runs
+ * enough: sequences then run one launch each; with that of the batch three to
+ * eight of them share their reads, each with the same bits).  The sum over the kept neurons runs
  * in list order split over the CTAs, so y agrees with clada_sparse_ffn_decode to
  * rounding (fp32 sums in another order), not bit for bit.  count_out [B] or
  * NULL receives the kept count.  A level outside 0..3, a count outside
