@@ -46,34 +46,30 @@ def rel_inf(a: np.ndarray, ref: np.ndarray) -> float:
 
 
 def launches(fn):
-    """[(kernel name, grid)] of the library's kernels that `fn` launches, in order, from a profiler trace.  A trace may lack
-    events: taken again until two agree; where none does the test is skipped."""
-    import json
-    import os
-    import tempfile
+    """[(kernel name, grid)] of the library's kernels that `fn` launches, in order: the kernel nodes of a CUDA graph that
+    captures the call."""
+    import subprocess
 
-    import pytest
-    from torch.profiler import ProfilerActivity, profile
+    from cuda.bindings import driver
 
-    def trace():
-        with profile(activities=[ProfilerActivity.CUDA]) as prof:
-            torch.cuda.synchronize()
-            fn()
-            torch.cuda.synchronize()
-        fd, path = tempfile.mkstemp(suffix=".json")
-        os.close(fd)
-        prof.export_chrome_trace(path)
-        with open(path) as f:
-            events = [e for e in json.load(f)["traceEvents"] if e.get("cat") == "kernel" and "clada::" in e["name"]]
-        os.remove(path)
-        return [(e["name"], tuple(e["args"]["grid"])) for e in sorted(events, key=lambda e: e["ts"])]
+    def get(result):
+        assert int(result[0]) == 0, result[0]
+        return result[1]
 
     fn()
     torch.cuda.synchronize()
-    seen = []
-    for _ in range(8):
-        ran = trace()
-        if ran and ran in seen:
-            return ran
-        seen.append(ran)
-    pytest.skip("the profiler's traces do not agree")
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        fn()
+    raw = graph.raw_cuda_graph()
+    n = driver.cuGraphGetNodes(raw, 0)
+    assert int(n[0]) == 0, n[0]
+    ran = []
+    for node in get(driver.cuGraphGetNodes(raw, n[2]))[:n[2]]:
+        if get(driver.cuGraphNodeGetType(node)) != driver.CUgraphNodeType.CU_GRAPH_NODE_TYPE_KERNEL:
+            continue
+        k = get(driver.cuGraphKernelNodeGetParams(node))
+        name = get(driver.cuFuncGetName(k.func) if int(k.func) else driver.cuKernelGetName(k.kern)).decode()
+        ran.append((name, (k.gridDimX, k.gridDimY, k.gridDimZ)))
+    names = subprocess.run(["c++filt"], input="\n".join(n for n, _ in ran), capture_output=True, text=True, check=True)
+    return [(n, grid) for n, (_, grid) in zip(names.stdout.splitlines(), ran) if "clada::" in n]
