@@ -257,7 +257,10 @@ sparse_ffn_kernel(const FfnParams p, const int n_stages) {
             else
                 reinterpret_cast<uint2 *>(p.y)[q] = make_uint2(0u, 0u);
         }
-        if (tid == 0) grid_leave(p.ctrl, (unsigned)n_ctas);
+        if (tid == 0) {
+            __threadfence();  // the count in grid_enter lands before the last CTA's departure clears it
+            grid_leave(p.ctrl, (unsigned)n_ctas);
+        }
         return;
     }
     __syncthreads();  // s_list and the mbarriers are ready

@@ -60,7 +60,8 @@ __device__ __forceinline__ bool grid_all_started(WsCtrl *ctrl, unsigned n_ctas) 
     asm volatile("ld.relaxed.gpu.u32 %0, [%1];" : "=r"(seen) : "l"(&ctrl->started) : "memory");
     return seen >= n_ctas;
 }
-// grid_leave: one thread of every CTA, once the CTA has nothing more to read from the control words.
+// grid_leave: one thread of every CTA, once the CTA has nothing more to read from the control words; between it and
+// grid_enter lies a device-wide fence (grid_meet has one), or a late count could land after the last CTA's reset.
 __device__ __forceinline__ void grid_leave(WsCtrl *ctrl, unsigned n_ctas) {
     const unsigned left = atomicAdd(&ctrl->depart, 1u);
     if (left == n_ctas - 1) {

@@ -22,12 +22,12 @@ def _layer(clada, d, F, dtype):
 
 
 class _Decode:
-    def __init__(self, clada, B, d, F, dtype, nested):
+    def __init__(self, clada, B, d, F, dtype, nested, tau=0.8):
         self.clada, self.layer, self.nested = clada, _layer(clada, d, F, dtype), nested
         g = torch.Generator(device="cuda").manual_seed(B)
         self.x = torch.randn(B, d, generator=g, device="cuda").to(dtype)
         self.scores = torch.rand(B, F, generator=g, device="cuda") + 0.5
-        self.tau = torch.full((B,), 0.8, device="cuda")
+        self.tau = torch.full((B,), tau, device="cuda")
         self.order = torch.empty(B, F, dtype=torch.int32, device="cuda")
         self.counts = torch.empty(B, 4, dtype=torch.int32, device="cuda")
         clada.clada_nested_build(self.scores, self.tau, 0.25, 0.1, self.order, self.counts)
@@ -50,6 +50,7 @@ class _Decode:
 FORMS = [(1, 1024, 2400, torch.bfloat16, False), (1, 512, 1376, torch.float32, False), (2, 1024, 2400, torch.bfloat16, False),
          (2, 512, 1376, torch.float32, False), (4, 512, 1376, torch.float32, False), (6, 1024, 2400, torch.float16, False),
          (20, 1024, 2400, torch.bfloat16, False), (1, 1024, 2400, torch.bfloat16, True), (5, 1024, 2400, torch.bfloat16, True)]
+NOTHING_KEPT = [(1, 1024, 2400, torch.bfloat16, False, 9.0), (1, 512, 1376, torch.float32, True, 9.0)]
 
 
 @pytest.mark.parametrize("B,d,F,dtype,nested", FORMS)
@@ -93,3 +94,25 @@ def test_two_streams(clada, first):
         assert decs[i].clean()
         for y in outs[i]:
             assert torch.equal(y, want[i])
+
+
+@pytest.mark.parametrize("form", NOTHING_KEPT)
+def test_launches_that_keep_nothing(clada, form):
+    """They leave without a meeting: y is zero, and the control words are zero for the dense pass behind each, which
+    numbers its CTAs by one of them.  On two streams, so that launches begin a few CTAs at a time."""
+    none, dense = [_Decode(clada, *form) for _ in (0, 1)], [_Decode(clada, 6, 1024, 2400, torch.bfloat16, False) for _ in (0, 1)]
+    want = dense[0].run()
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    for i in (0, 1):
+        none[i].ws = dense[i].ws  # one workspace for both kinds
+    torch.cuda.synchronize()
+    outs = []
+    for _ in range(40):
+        for i in (0, 1):
+            with torch.cuda.stream(streams[i]):
+                outs.append((none[i].run(), dense[i].run()))
+    torch.cuda.synchronize()
+    for i in (0, 1):
+        assert none[i].clean() and dense[i].clean()
+    for zero, y in outs:
+        assert torch.all(zero == 0) and torch.equal(y, want)
