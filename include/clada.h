@@ -124,6 +124,19 @@ int clada_stream_read_probe(const void *buf, size_t bytes, uint32_t *sink, void 
 int clada_selftest_bounded_waits(void *ws, size_t ws_bytes, uint32_t poll_limit, int32_t *report,
                                  int32_t *status, void *stream);
 
+/* Self-test of the decode launches' meeting (the paper has no counterpart).  Their
+ * CTAs need not be resident together: one that comes to the meeting before all
+ * have begun leaves, and those that come later share its part of the final sums.
+ * This call takes n_ctas CTAs (1 .. 64) through a meeting in which the last n_late
+ * begin after the others have come: those leave, the n_late share all parts (0: all
+ * wait, each has its own part).  n_late = -1: none waits, the last one to come
+ * does everything.
+ *   report      out [n_ctas][2] int32, device: part and number of parts of each CTA
+ *               (0 parts: it left; -1: a wait gave up, and status has CLADA_STATUS_TIMEOUT)
+ * The workspace's control words are zero before and after. */
+int clada_selftest_meeting(void *ws, size_t ws_bytes, int32_t n_ctas, int32_t n_late, int32_t *report,
+                           int32_t *status, void *stream);
+
 /* out[j] = ||W_out,j||_2 = the l2 norm of row j of w_down_t, fp32.  Once per
  * layer; the second factor of Eq. neuron_activation. */
 int clada_down_norms(const clada_layer *layer, float *out /*[d_ff]*/, void *stream);

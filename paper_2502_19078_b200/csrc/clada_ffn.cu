@@ -324,16 +324,15 @@ sparse_ffn_kernel(const FfnParams p, const int n_stages) {
     if (timed_out && p.status) atomicOr(p.status, CLADA_STATUS_TIMEOUT);
 
     // ---- epilogue: the CTAs meet, deterministic column reduction --------------------------------
-    const GridMeet how = grid_meet(p.ctrl, (unsigned)n_ctas, kConsumers, &s_all);
-    if (how == kMeetTimeout && tid == 0 && p.status) atomicOr(p.status, CLADA_STATUS_TIMEOUT);
-    if (how == kMeetTimeout || how == kMeetLeave) return;
-    const int q_first = how == kMeetWhole ? warp : cta + warp * n_ctas, q_step = how == kMeetWhole ? kFfnWarps : n_ctas * kFfnWarps;
+    const GridPart mine = grid_meet(p.ctrl, (unsigned)n_ctas, cta, kConsumers, &s_all);
+    if (mine.parts < 0 && tid == 0 && p.status) atomicOr(p.status, CLADA_STATUS_TIMEOUT);
+    if (mine.parts <= 0) return;
     // columns in groups of 4 (float4); a warp sums one group: lane l adds partial rows l, l+32, ... (one row
     // per CTA and consumer group) in order (five loads in flight at a time), then the 32 lane sums combine by
     // butterfly.
     const int ngroups = d / 4;
     const int n_rows = n_ctas * GROUPS;
-    for (int q = q_first; q < ngroups; q += q_step) {
+    for (int q = mine.part + warp * mine.parts; q < ngroups; q += mine.parts * kFfnWarps) {
         float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
         for (int rb = 0; rb < n_rows; rb += 5 * kWarp) {
             float4 v[5];

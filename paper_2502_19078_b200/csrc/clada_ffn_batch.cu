@@ -253,10 +253,10 @@ sparse_ffn_batch_kernel(const FfnBatchParams p, const int n_stages) {
     if (timed_out && p.status) atomicOr(p.status, CLADA_STATUS_TIMEOUT);
 
     // ---- epilogue: the CTAs meet, deterministic column reduction per sequence --------------------
-    const GridMeet how = grid_meet(p.ctrl, (unsigned)n_ctas, kConsumers, &s_all);
-    if (how == kMeetTimeout && tid == 0 && p.status) atomicOr(p.status, CLADA_STATUS_TIMEOUT);
-    if (how == kMeetTimeout || how == kMeetLeave) return;
-    batch_column_sums<BT>(p, how == kMeetWhole);
+    const GridPart mine = grid_meet(p.ctrl, (unsigned)n_ctas, cta, kConsumers, &s_all);
+    if (mine.parts < 0 && tid == 0 && p.status) atomicOr(p.status, CLADA_STATUS_TIMEOUT);
+    if (mine.parts <= 0) return;
+    batch_column_sums<BT>(p, mine);
 }
 
 

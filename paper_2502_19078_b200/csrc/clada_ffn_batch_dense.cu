@@ -568,17 +568,16 @@ sparse_ffn_batch_dense_kernel(const __grid_constant__ CUtensorMap map_x, const _
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kBdTmemCols) : "memory");
     }
     // ---- all groups' partial outputs are in global memory after the meeting: sum them in group order ----------
-    const GridMeet how = grid_meet(p.ctrl, gridDim.x, 32, &s_all);
-    if (how == kMeetTimeout && threadIdx.x == 0 && p.status) atomicOr(p.status, CLADA_STATUS_TIMEOUT);
-    if (how == kMeetTimeout || how == kMeetLeave) return;
+    const GridPart mine = grid_meet(p.ctrl, gridDim.x, cta, 32, &s_all);
+    if (mine.parts < 0 && threadIdx.x == 0 && p.status) atomicOr(p.status, CLADA_STATUS_TIMEOUT);
+    if (mine.parts <= 0) return;
     if (threadIdx.x == 0) BD_TRACE(12);
-    const bool whole = how == kMeetWhole;
-    if ((cta == 0 || whole) && threadIdx.x < 64 - kBdGroupWord0)  // every member has passed its group's counter: clear them
+    if (mine.part == 0 && threadIdx.x < 64 - kBdGroupWord0)  // every member has passed its group's counter: clear them
         reinterpret_cast<unsigned *>(p.ctrl)[kBdGroupWord0 + threadIdx.x] = 0u;
     const int d4 = p.d_model / 4;
-    // every CTA takes an equal run of (sequence, four columns)
-    const int share = whole ? p.B * d4 : (p.B * d4 + gridDim.x - 1) / gridDim.x;
-    const int it0 = whole ? 0 : cta * share, it1 = min(p.B * d4, it0 + share);
+    // a part is an equal run of (sequence, four columns)
+    const int share = (p.B * d4 + mine.parts - 1) / mine.parts;
+    const int it0 = mine.part * share, it1 = min(p.B * d4, it0 + share);
     for (int it = it0 + threadIdx.x; it < it1; it += kBdThreads) {
         const int b = it / d4, q = it - b * d4;
         float4 s = make_float4(0.f, 0.f, 0.f, 0.f);

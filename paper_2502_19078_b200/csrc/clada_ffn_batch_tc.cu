@@ -331,11 +331,11 @@ sparse_ffn_batch_tc_kernel(const FfnBatchParams p, const int n_slots) {
     TC_TRACE(255, 4);
 
     // ---- epilogue: the CTAs meet, deterministic column reduction per sequence --------------------
-    const GridMeet how = grid_meet(p.ctrl, (unsigned)n_ctas, kWarp, &s_all);
-    if (how == kMeetTimeout && tid == 0 && p.status) atomicOr(p.status, CLADA_STATUS_TIMEOUT);
-    if (how == kMeetTimeout || how == kMeetLeave) return;
+    const GridPart mine = grid_meet(p.ctrl, (unsigned)n_ctas, cta, kWarp, &s_all);
+    if (mine.parts < 0 && tid == 0 && p.status) atomicOr(p.status, CLADA_STATUS_TIMEOUT);
+    if (mine.parts <= 0) return;
     TC_TRACE(255, 5);
-    batch_column_sums<BT, kConsumers>(p, how == kMeetWhole);
+    batch_column_sums<BT, kConsumers>(p, mine);
     TC_TRACE(255, 6);
 }
 

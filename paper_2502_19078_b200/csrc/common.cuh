@@ -44,6 +44,7 @@ struct WsCtrl {
     unsigned int arrive;  // grid barrier: CTAs that reached it
     unsigned int depart;  // CTAs that left it; the last one resets all of these
     unsigned int started; // CTAs that have begun (grid_enter)
+    unsigned int shared;  // parts taken over from CTAs that did not wait (grid_meet)
 };
 
 // ---- device helpers -----------------------------------------------------------------------

@@ -141,15 +141,14 @@ __device__ __forceinline__ int batch_union_share(const FfnBatchParams &p, const 
     return r1 - r0;
 }
 
-// Epilogue of a tile: after the meeting every CTA sums a slice (whole: all) of the (sequence, column group) pairs over all
+// Epilogue of a tile: after the meeting a CTA sums its part of the (sequence, column group) pairs over all
 // CTAs' partial rows [n_ctas][BT][d_model] in CTA order (a warp per group of 4 columns: lane l adds rows l,
 // l+32, ..., then the 32 lane sums combine by butterfly) and writes y.
 template <int BT, int NT = kFfnThreads>
-__device__ __forceinline__ void batch_column_sums(const FfnBatchParams &p, const bool whole) {
+__device__ __forceinline__ void batch_column_sums(const FfnBatchParams &p, const GridPart mine) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int cta = blockIdx.x, n_ctas = gridDim.x, d = p.d_model;
-    const int ngroups = d / 4, step = whole ? NT / kWarp : n_ctas * (NT / kWarp);
-    for (int it = whole ? warp : cta + warp * n_ctas; it < BT * ngroups; it += step) {
+    const int n_ctas = gridDim.x, d = p.d_model, ngroups = d / 4;
+    for (int it = mine.part + warp * mine.parts; it < BT * ngroups; it += mine.parts * (NT / kWarp)) {
         const int b = it / ngroups, q = it % ngroups;
         float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
         for (int rb = 0; rb < n_ctas; rb += 5 * kWarp) {

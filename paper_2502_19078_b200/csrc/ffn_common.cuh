@@ -46,10 +46,14 @@ static __device__ bool grid_barrier(WsCtrl *ctrl, unsigned n_ctas, int depart_ti
 
 // Grid-wide meeting of a plain launch, whose CTAs need not all be resident at once.  A cooperative launch begins only
 // after its predecessor has left the SMs; a plain one has its CTAs in place (barriers set up, in griddepcontrol.wait)
-// when the predecessor ends.  What must not happen is that a CTA waits for one that the scheduler has not placed: so a
-// CTA waits only if it has seen that all CTAs have begun, for then every one of them reaches the meeting by itself.
-// Otherwise it counts itself in as not waiting and leaves, and the CTA that comes last does everybody's part.  (Two such
-// launches on different streams may hold half of the SMs each: both then end this way.)
+// when the predecessor ends.  At the meeting no CTA waits for one that the scheduler has not placed: a CTA waits only if it
+// has seen that all CTAs have begun, for then every one of them comes by itself.  Otherwise it counts itself in as not
+// waiting and leaves, and those that do wait share its part; if nobody waits, the CTA that comes last does every part.
+// (Two such launches on different streams may hold half of the SMs each: both then end this way.)  Decodes on one stream
+// beside prompts of 96 tokens on another (112 CTAs each), us a decode and a prompt, cooperative / all parts by the last CTA /
+// shared: one sequence of 4096 x 11008 60 + 87, 81 + 121, 47 + 87; two of 2560 x 10240 61 + 85, 121 + 156, 49 + 85; four of
+// 1024 x 4096 fp32 53 + 79, 92 + 127, 44 + 79; 8 of 4096 x 14336 90 + 117, 113 + 139, 89 + 116; 32 of 5120 x 13824 110 + 136,
+// 101 + 136, 101 + 137.
 // Measured (us a decode step, cooperative / plain): 512 x 1376 fp32 14.8 / 13.9, 1024 x 4100 19.8 / 18.2, 4096 x 11008 39.8 /
 // 38.3, two sequences of 2560 x 10240 31.2 / 29.8, 8 of 4096 x 14336 71.8 / 69.4, 32 of 5120 x 13824 93.2 / 92.0.
 // grid_enter: one thread, after pdl_wait() (the control words may be the predecessor's until then); returns how many CTAs
@@ -68,40 +72,52 @@ __device__ __forceinline__ void grid_leave(WsCtrl *ctrl, unsigned n_ctas) {
         ctrl->arrive = 0;
         ctrl->depart = 0;
         ctrl->started = 0;
+        ctrl->shared = 0;
         __threadfence();
     }
 }
-enum GridMeet { kMeetSlice, kMeetWhole, kMeetLeave, kMeetTimeout };  // do your own part, do every part, none, gave up
-constexpr unsigned kMeetCount = 0xffffu, kMeetNoWait = 0x10000u;     // arrive: CTAs that came, and above them those that did not wait
-// s_all: shared word, non-zero if some thread of the CTA has already seen that all CTAs have begun.
-static __device__ GridMeet grid_meet(WsCtrl *ctrl, unsigned n_ctas, int depart_tid, const int *s_all) {
-    __shared__ int s_how;
+// What is left for a CTA to do after the meeting: part `part` of `parts` equal ones; nothing (0 parts: it left, others do
+// it); or the wait gave up (parts < 0).
+struct GridPart {
+    int part, parts;
+};
+constexpr unsigned kMeetCount = 0xffffu, kMeetNoWait = 0x10000u;  // arrive: CTAs that came, and above them those that did not wait
+// cta: this CTA's part when all wait.  s_all: shared word, non-zero if some thread of the CTA has already seen that all CTAs
+// have begun (null: this CTA does not wait).
+static __device__ GridPart grid_meet(WsCtrl *ctrl, unsigned n_ctas, int cta, int depart_tid, const int *s_all) {
+    __shared__ int s_part, s_parts;
     __syncthreads();
     if (threadIdx.x == 0) {
-        const bool wait = *s_all != 0 || grid_all_started(ctrl, n_ctas);
+        const bool wait = s_all && (*s_all != 0 || grid_all_started(ctrl, n_ctas));
         const unsigned mine = wait ? 1u : 1u + kMeetNoWait;
         __threadfence();
-        const unsigned came = atomicAdd(&ctrl->arrive, mine) + mine;
-        int how = came >= kMeetNoWait ? kMeetWhole : kMeetSlice;
-        if ((came & kMeetCount) != n_ctas) {  // not the last one
-            how = wait ? kMeetSlice : kMeetLeave;
-            unsigned spins = 0, seen = 0;
-            while (wait) {
-                asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(seen) : "l"(&ctrl->arrive) : "memory");
-                if ((seen & kMeetCount) >= n_ctas) break;
+        unsigned seen = atomicAdd(&ctrl->arrive, mine) + mine;
+        int part = cta, parts = (int)n_ctas;
+        if (!wait) {
+            part = 0;
+            parts = seen == n_ctas * (1u + kMeetNoWait) ? 1 : 0;  // the last one, and all have left
+        } else {
+            unsigned spins = 0;
+            while ((seen & kMeetCount) < n_ctas) {
                 if (++spins > kBarrierSpinLimit) {
-                    how = kMeetTimeout;
+                    parts = -1;
                     break;
                 }
+                asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(seen) : "l"(&ctrl->arrive) : "memory");
+            }
+            if (parts > 0 && seen >= kMeetNoWait) {
+                parts = (int)(n_ctas - seen / kMeetNoWait);
+                part = (int)atomicAdd(&ctrl->shared, 1u);
             }
         }
         __threadfence();
-        s_how = how;
+        s_part = part;
+        s_parts = parts;
     }
     __syncthreads();
-    const GridMeet how = static_cast<GridMeet>(s_how);
-    if ((int)threadIdx.x == depart_tid && how != kMeetTimeout) grid_leave(ctrl, n_ctas);
-    return how;
+    const GridPart mine = {s_part, s_parts};
+    if ((int)threadIdx.x == depart_tid && mine.parts >= 0) grid_leave(ctrl, n_ctas);
+    return mine;
 }
 
 // ---- mbarrier / bulk-copy primitives (bounded waits) -------------------------------------------

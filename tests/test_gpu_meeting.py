@@ -116,3 +116,23 @@ def test_launches_that_keep_nothing(clada, form):
         assert none[i].clean() and dense[i].clean()
     for zero, y in outs:
         assert torch.all(zero == 0) and torch.equal(y, want)
+
+
+@pytest.mark.parametrize("n,late", [(1, 0), (1, 1), (5, 0), (5, 5), (5, 2), (64, 1), (64, 40), (64, 63), (1, -1), (64, -1)])
+def test_parts_of_a_meeting(clada, n, late):
+    """Who leaves and who does what, with CTAs made to begin late: no part is lost and none is done twice, the parts of
+    CTAs that left are shared by all that came later, and a meeting that everybody left is the last one's alone."""
+    ws = torch.zeros(256, dtype=torch.uint8, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for _ in range(20):
+        report = torch.full((n, 2), -9, dtype=torch.int32, device="cuda")
+        clada.clada_selftest_meeting(ws, n, late, report, status)
+        got = report.tolist()
+        if late < 0:
+            assert sorted(got) == [[0, 0]] * (n - 1) + [[0, 1]]
+        elif late in (0, n):
+            assert got == [[c, n] for c in range(n)]
+        else:
+            assert [parts for _, parts in got[:n - late]] == [0] * (n - late)
+            assert sorted(got[n - late:]) == [[c, late] for c in range(late)]
+        assert int(status.item()) == 0 and int(ws.view(torch.int32).abs().sum().item()) == 0
