@@ -128,9 +128,8 @@ int clada_selftest_bounded_waits(void *ws, size_t ws_bytes, uint32_t poll_limit,
  * CTAs need not be resident together: one that comes to the meeting before all
  * have begun leaves, and those that come later share its part of the final sums.
  * This call takes n_ctas CTAs (1 .. 64) through a meeting in which the last n_late
- * begin after the others have come: those leave, the n_late share all parts (0: all
- * wait, each has its own part).  n_late = -1: none waits, the last one to come
- * does everything.
+ * begin after the others have come and left: the n_late share all parts (0: all
+ * wait, each has its own part).
  *   report      out [n_ctas][2] int32, device: part and number of parts of each CTA
  *               (0 parts: it left; -1: a wait gave up, and status has CLADA_STATUS_TIMEOUT)
  * The workspace's control words are zero before and after. */

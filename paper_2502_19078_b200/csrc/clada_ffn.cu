@@ -69,10 +69,8 @@ sparse_ffn_kernel(const FfnParams p, const int n_stages) {
         mbar_init(sbar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    __shared__ int s_all;  // every CTA of the launch has begun
-    if (tid == 0) s_all = 0;
     pdl_wait();  // everything below may read what the previous kernel wrote
-    if (tid == 0) grid_enter(p.ctrl);
+    if (tid == kConsumers + 1) grid_enter(p.ctrl);  // a thread with nothing else to do
 
     const uint64_t keep_policy = policy_evict_last();
     const bool nested = p.order != nullptr;
@@ -294,7 +292,6 @@ sparse_ffn_kernel(const FfnParams p, const int n_stages) {
                     par ^= 1;
                 }
             }
-            if (grid_all_started(p.ctrl, (unsigned)n_ctas)) s_all = 1;
             // Never leave with copies in flight: the last use of every stage must have landed.
             for (int i = max(0, issued - n_stages); i < issued; ++i)
                 if (!mbar_wait(full0 + 8 * (i % n_stages), (i / n_stages) & 1)) timed_out = true;
@@ -324,7 +321,7 @@ sparse_ffn_kernel(const FfnParams p, const int n_stages) {
     if (timed_out && p.status) atomicOr(p.status, CLADA_STATUS_TIMEOUT);
 
     // ---- epilogue: the CTAs meet, deterministic column reduction --------------------------------
-    const GridPart mine = grid_meet(p.ctrl, (unsigned)n_ctas, cta, kConsumers, &s_all);
+    const GridPart mine = grid_meet(p.ctrl, (unsigned)n_ctas, cta, kConsumers);
     if (mine.parts < 0 && tid == 0 && p.status) atomicOr(p.status, CLADA_STATUS_TIMEOUT);
     if (mine.parts <= 0) return;
     // columns in groups of 4 (float4); a warp sums one group: lane l adds partial rows l, l+32, ... (one row

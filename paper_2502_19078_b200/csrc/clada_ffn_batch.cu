@@ -55,8 +55,6 @@ sparse_ffn_batch_kernel(const FfnBatchParams p, const int n_stages) {
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    __shared__ int s_all;  // every CTA of the launch has begun
-    if (tid == 0) s_all = 0;
     pdl_wait();
     if (tid == 0) grid_enter(p.ctrl);
 
@@ -109,7 +107,6 @@ sparse_ffn_batch_kernel(const FfnBatchParams p, const int n_stages) {
                     par ^= 1;
                 }
             }
-            if (grid_all_started(p.ctrl, (unsigned)n_ctas)) s_all = 1;
             for (int i = max(0, issued - n_stages); i < issued; ++i)
                 if (!mbar_wait(full0 + 8 * (i % n_stages), (i / n_stages) & 1)) timed_out = true;
         }
@@ -253,7 +250,7 @@ sparse_ffn_batch_kernel(const FfnBatchParams p, const int n_stages) {
     if (timed_out && p.status) atomicOr(p.status, CLADA_STATUS_TIMEOUT);
 
     // ---- epilogue: the CTAs meet, deterministic column reduction per sequence --------------------
-    const GridPart mine = grid_meet(p.ctrl, (unsigned)n_ctas, cta, kConsumers, &s_all);
+    const GridPart mine = grid_meet(p.ctrl, (unsigned)n_ctas, cta, kConsumers);
     if (mine.parts < 0 && tid == 0 && p.status) atomicOr(p.status, CLADA_STATUS_TIMEOUT);
     if (mine.parts <= 0) return;
     batch_column_sums<BT>(p, mine);

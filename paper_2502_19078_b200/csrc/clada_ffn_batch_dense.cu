@@ -193,7 +193,7 @@ sparse_ffn_batch_dense_kernel(const __grid_constant__ CUtensorMap map_x, const _
     __shared__ __align__(8) uint64_t s_full[kBdMaxStages], s_empty[kBdMaxStages], s_p1_full, s_h_own, s_h_all,
         s_tile_full[kBdMaxTiles], s_tile_read[kBdMaxTiles];
     __shared__ uint32_t s_tmem_base;
-    __shared__ int s_abort, s_group_ok, s_cta, s_all;
+    __shared__ int s_abort, s_group_ok, s_cta;
 
     constexpr int kPer = SEQS / 2;  // sequences of an epilogue warp
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -221,7 +221,6 @@ sparse_ffn_batch_dense_kernel(const __grid_constant__ CUtensorMap map_x, const _
         }
         s_abort = 0;
         s_group_ok = 0;
-        s_all = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     // Rows rows_blk .. rpad-1 of every box slot are never written by a copy but are read by the last K step of
@@ -311,7 +310,6 @@ sparse_ffn_batch_dense_kernel(const __grid_constant__ CUtensorMap map_x, const _
             }
             BD_TRACE(15);
             if (!ok) *abort_flag = 1;
-            if (grid_all_started(p.ctrl, gridDim.x)) s_all = 1;
             for (int i = max(0, kc - n_stages); i < kc; ++i) {  // never leave with copies in flight
                 int never = 0;
                 if (!tc_mbar_wait(tc_smem_u32(&s_full[i % n_stages]), (i / n_stages) & 1, &never)) *abort_flag = 1;
@@ -568,7 +566,7 @@ sparse_ffn_batch_dense_kernel(const __grid_constant__ CUtensorMap map_x, const _
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kBdTmemCols) : "memory");
     }
     // ---- all groups' partial outputs are in global memory after the meeting: sum them in group order ----------
-    const GridPart mine = grid_meet(p.ctrl, gridDim.x, cta, 32, &s_all);
+    const GridPart mine = grid_meet(p.ctrl, gridDim.x, cta, 32);
     if (mine.parts < 0 && threadIdx.x == 0 && p.status) atomicOr(p.status, CLADA_STATUS_TIMEOUT);
     if (mine.parts <= 0) return;
     if (threadIdx.x == 0) BD_TRACE(12);

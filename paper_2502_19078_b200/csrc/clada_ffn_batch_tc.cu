@@ -126,8 +126,6 @@ sparse_ffn_batch_tc_kernel(const FfnBatchParams p, const int n_slots) {
         for (int s = 0; s < n_slots; ++s) mbar_init(full0 + 8 * s, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    __shared__ int s_all;  // every CTA of the launch has begun
-    if (tid == 0) s_all = 0;
     pdl_wait();
     if (tid == 0) grid_enter(p.ctrl);
     TC_TRACE(255, 0);
@@ -308,7 +306,6 @@ sparse_ffn_batch_tc_kernel(const FfnBatchParams p, const int n_slots) {
         TC_TRACE(g0 / CH, 6);
     }
     TC_TRACE(255, 3);
-    if (tid == kWarp && grid_all_started(p.ctrl, (unsigned)n_ctas)) s_all = 1;
     // Never leave with copies in flight.  Every copy issued was waited for above, unless a wait gave up: then
     // thread 0 waits (bounded again) for the last slots' worth.
     if (timed_out && tid == 0) {
@@ -331,7 +328,7 @@ sparse_ffn_batch_tc_kernel(const FfnBatchParams p, const int n_slots) {
     TC_TRACE(255, 4);
 
     // ---- epilogue: the CTAs meet, deterministic column reduction per sequence --------------------
-    const GridPart mine = grid_meet(p.ctrl, (unsigned)n_ctas, cta, kWarp, &s_all);
+    const GridPart mine = grid_meet(p.ctrl, (unsigned)n_ctas, cta, kWarp);
     if (mine.parts < 0 && tid == 0 && p.status) atomicOr(p.status, CLADA_STATUS_TIMEOUT);
     if (mine.parts <= 0) return;
     TC_TRACE(255, 5);

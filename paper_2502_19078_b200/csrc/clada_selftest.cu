@@ -31,23 +31,22 @@ bounded_wait_selftest_kernel(WsCtrl *ctrl, unsigned poll_limit, int32_t *report,
 }
 
 // The meeting with CTAs that begin late, as where other work holds SMs: of n CTAs the last n_late begin only after the others
-// have come to the meeting (which therefore leave it), and come themselves once all have begun.  n_late < 0: nobody waits.
+// have come to the meeting and left it, and come themselves once all have begun.
 __global__ void __launch_bounds__(64, 1)
 meeting_selftest_kernel(WsCtrl *ctrl, int n_late, int32_t *report, int32_t *status) {
-    __shared__ int s_all;
     const unsigned n = gridDim.x, cta = blockIdx.x;
     const unsigned early = n_late > 0 ? n - (unsigned)n_late : 0u;  // n_late 0: all begin, then all come
     if (threadIdx.x == 0) {
-        unsigned seen = 0;
-        s_all = 0;
-        if (cta >= early && early > 0)
-            for (unsigned i = 0; i < kBarrierSpinLimit && (seen & kMeetCount) < early; ++i)
+        unsigned seen = 0, begun = 0;
+        if (cta >= early)
+            for (unsigned i = 0; i < kBarrierSpinLimit && seen / kMeetLeft < early; ++i)
                 asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(seen) : "l"(&ctrl->arrive) : "memory");
         grid_enter(ctrl);
-        if (cta >= early && n_late >= 0)
-            for (unsigned i = 0; i < kBarrierSpinLimit && s_all == 0; ++i) s_all = grid_all_started(ctrl, n) ? 1 : 0;
+        if (cta >= early)
+            for (unsigned i = 0; i < kBarrierSpinLimit && begun < n; ++i)
+                asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(begun) : "l"(&ctrl->started) : "memory");
     }
-    const GridPart mine = grid_meet(ctrl, n, (int)cta, 32, n_late < 0 ? nullptr : &s_all);
+    const GridPart mine = grid_meet(ctrl, n, (int)cta, 32);
     if (threadIdx.x == 0) {
         report[2 * cta] = mine.part;
         report[2 * cta + 1] = mine.parts;
@@ -63,7 +62,7 @@ extern "C" int clada_selftest_meeting(void *ws, size_t ws_bytes, int32_t n_ctas,
                                       int32_t *status, void *stream) {
     if (!ws || !report) return CLADA_ERR_NULL;
     if (ws_bytes < kWsCtrlBytes || (reinterpret_cast<uintptr_t>(ws) & 255u)) return CLADA_ERR_WORKSPACE;
-    if (n_ctas < 1 || n_ctas > 64 || n_late < -1 || n_late > n_ctas) return CLADA_ERR_SHAPE;  // 64: resident together
+    if (n_ctas < 1 || n_ctas > 64 || n_late < 0 || n_late > n_ctas) return CLADA_ERR_SHAPE;  // 64: resident together
     meeting_selftest_kernel<<<n_ctas, 64, 0, static_cast<cudaStream_t>(stream)>>>(static_cast<WsCtrl *>(ws), n_late, report, status);
     CLADA_CUDA_TRY(cudaGetLastError());
     return CLADA_OK;

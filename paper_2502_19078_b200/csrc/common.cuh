@@ -40,11 +40,11 @@ int device_info(DeviceInfo *out);
 // [0, 256)            control words (grid-barrier counters), zeroed by clada_workspace_init
 // [256, ...)          per-call scratch
 constexpr size_t kWsCtrlBytes = 256;
-struct WsCtrl {
-    unsigned int arrive;  // grid barrier: CTAs that reached it
-    unsigned int depart;  // CTAs that left it; the last one resets all of these
-    unsigned int started; // CTAs that have begun (grid_enter)
-    unsigned int shared;  // parts taken over from CTAs that did not wait (grid_meet)
+struct alignas(16) WsCtrl {
+    unsigned int arrive;  // CTAs that came to the meeting (and, from bit 16 on, those of them that left at once)
+    unsigned int started; // CTAs that have begun; grid_enter and grid_meet take both words as one of 64 bits
+    unsigned int depart;  // CTAs that are through; the last one resets all of these
+    unsigned int shared;  // parts taken over from CTAs that left (grid_meet)
 };
 
 // ---- device helpers -----------------------------------------------------------------------

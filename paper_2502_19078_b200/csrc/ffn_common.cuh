@@ -47,8 +47,8 @@ static __device__ bool grid_barrier(WsCtrl *ctrl, unsigned n_ctas, int depart_ti
 // Grid-wide meeting of a plain launch, whose CTAs need not all be resident at once.  A cooperative launch begins only
 // after its predecessor has left the SMs; a plain one has its CTAs in place (barriers set up, in griddepcontrol.wait)
 // when the predecessor ends.  At the meeting no CTA waits for one that the scheduler has not placed: a CTA waits only if it
-// has seen that all CTAs have begun, for then every one of them comes by itself.  Otherwise it counts itself in as not
-// waiting and leaves, and those that do wait share its part; if nobody waits, the CTA that comes last does every part.
+// has seen that all CTAs have begun, for then every one of them comes by itself.  Otherwise it notes that it leaves, and
+// those that wait (at least the one that comes last) share its part.
 // (Two such launches on different streams may hold half of the SMs each: both then end this way.)  Decodes on one stream
 // beside prompts of 96 tokens on another (112 CTAs each), us a decode and a prompt, cooperative / all parts by the last CTA /
 // shared: one sequence of 4096 x 11008 60 + 87, 81 + 121, 47 + 87; two of 2560 x 10240 61 + 85, 121 + 156, 49 + 85; four of
@@ -58,21 +58,15 @@ static __device__ bool grid_barrier(WsCtrl *ctrl, unsigned n_ctas, int depart_ti
 // 38.3, two sequences of 2560 x 10240 31.2 / 29.8, 8 of 4096 x 14336 71.8 / 69.4, 32 of 5120 x 13824 93.2 / 92.0.
 // grid_enter: one thread, after pdl_wait() (the control words may be the predecessor's until then); returns how many CTAs
 // began before this one.
-__device__ __forceinline__ unsigned grid_enter(WsCtrl *ctrl) { return atomicAdd(&ctrl->started, 1u); }
-__device__ __forceinline__ bool grid_all_started(WsCtrl *ctrl, unsigned n_ctas) {
-    unsigned seen;
-    asm volatile("ld.relaxed.gpu.u32 %0, [%1];" : "=r"(seen) : "l"(&ctrl->started) : "memory");
-    return seen >= n_ctas;
+__device__ __forceinline__ unsigned grid_enter(WsCtrl *ctrl) {
+    return (unsigned)(atomicAdd(reinterpret_cast<unsigned long long *>(ctrl), 1ull << 32) >> 32);
 }
 // grid_leave: one thread of every CTA, once the CTA has nothing more to read from the control words; between it and
 // grid_enter lies a device-wide fence (grid_meet has one), or a late count could land after the last CTA's reset.
 __device__ __forceinline__ void grid_leave(WsCtrl *ctrl, unsigned n_ctas) {
     const unsigned left = atomicAdd(&ctrl->depart, 1u);
     if (left == n_ctas - 1) {
-        ctrl->arrive = 0;
-        ctrl->depart = 0;
-        ctrl->started = 0;
-        ctrl->shared = 0;
+        *reinterpret_cast<uint4 *>(ctrl) = make_uint4(0u, 0u, 0u, 0u);
         __threadfence();
     }
 }
@@ -81,36 +75,41 @@ __device__ __forceinline__ void grid_leave(WsCtrl *ctrl, unsigned n_ctas) {
 struct GridPart {
     int part, parts;
 };
-constexpr unsigned kMeetCount = 0xffffu, kMeetNoWait = 0x10000u;  // arrive: CTAs that came, and above them those that did not wait
-// cta: this CTA's part when all wait.  s_all: shared word, non-zero if some thread of the CTA has already seen that all CTAs
-// have begun (null: this CTA does not wait).
-static __device__ GridPart grid_meet(WsCtrl *ctrl, unsigned n_ctas, int cta, int depart_tid, const int *s_all) {
+constexpr unsigned kMeetCount = 0xffffu, kMeetLeft = 0x10000u;  // arrive: CTAs that came; one that left at once
+// cta: this CTA's part when all wait.  The way of a launch that is alone on the device is an addition and a poll, as in a
+// plain barrier (a second fence behind the poll and the added word's return trip before it made FFN launches in a graph 8.8
+// us instead of @@@ on 512 x 1376 fp32, 13.3 instead of @@@ on 1024 x 4100, 34.5 instead of @@@ on 4096 x 11008).
+static __device__ GridPart grid_meet(WsCtrl *ctrl, unsigned n_ctas, int cta, int depart_tid,
+                                     unsigned spin_limit = kBarrierSpinLimit) {
     __shared__ int s_part, s_parts;
     __syncthreads();
     if (threadIdx.x == 0) {
-        const bool wait = s_all && (*s_all != 0 || grid_all_started(ctrl, n_ctas));
-        const unsigned mine = wait ? 1u : 1u + kMeetNoWait;
         __threadfence();
-        unsigned seen = atomicAdd(&ctrl->arrive, mine) + mine;
+        unsigned long long *word = reinterpret_cast<unsigned long long *>(ctrl);  // started << 32 | left << 16 | came
+        atomicAdd(word, 1ull);
         int part = cta, parts = (int)n_ctas;
-        if (!wait) {
-            part = 0;
-            parts = seen == n_ctas * (1u + kMeetNoWait) ? 1 : 0;  // the last one, and all have left
-        } else {
-            unsigned spins = 0;
-            while ((seen & kMeetCount) < n_ctas) {
-                if (++spins > kBarrierSpinLimit) {
-                    parts = -1;
-                    break;
+        unsigned spins = 0;
+        for (;;) {
+            unsigned long long seen;
+            asm volatile("ld.acquire.gpu.u64 %0, [%1];" : "=l"(seen) : "l"(word) : "memory");
+            if (((unsigned)seen & kMeetCount) >= n_ctas) {
+                const unsigned left = (unsigned)seen / kMeetLeft;
+                if (left > 0) {  // those that stayed share all parts
+                    parts = (int)(n_ctas - left);
+                    part = (int)atomicAdd(&ctrl->shared, 1u);
                 }
-                asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(seen) : "l"(&ctrl->arrive) : "memory");
+                break;
             }
-            if (parts > 0 && seen >= kMeetNoWait) {
-                parts = (int)(n_ctas - seen / kMeetNoWait);
-                part = (int)atomicAdd(&ctrl->shared, 1u);
+            // Leaving is noted only while somebody is still to come, so that all who wait see the same number.
+            if ((unsigned)(seen >> 32) < n_ctas && atomicCAS(word, seen, seen + kMeetLeft) == seen) {
+                part = parts = 0;
+                break;
+            }
+            if (++spins > spin_limit) {
+                parts = -1;
+                break;
             }
         }
-        __threadfence();
         s_part = part;
         s_parts = parts;
     }

@@ -118,19 +118,17 @@ def test_launches_that_keep_nothing(clada, form):
         assert torch.all(zero == 0) and torch.equal(y, want)
 
 
-@pytest.mark.parametrize("n,late", [(1, 0), (1, 1), (5, 0), (5, 5), (5, 2), (64, 1), (64, 40), (64, 63), (1, -1), (64, -1)])
+@pytest.mark.parametrize("n,late", [(1, 0), (1, 1), (5, 0), (5, 5), (5, 2), (64, 1), (64, 40), (64, 63)])
 def test_parts_of_a_meeting(clada, n, late):
-    """Who leaves and who does what, with CTAs made to begin late: no part is lost and none is done twice, the parts of
-    CTAs that left are shared by all that came later, and a meeting that everybody left is the last one's alone."""
+    """Who leaves and who does what, with CTAs made to begin late: no part is lost and none is done twice, and the parts of
+    CTAs that left are shared by all that came later."""
     ws = torch.zeros(256, dtype=torch.uint8, device="cuda")
     status = torch.zeros(1, dtype=torch.int32, device="cuda")
     for _ in range(20):
         report = torch.full((n, 2), -9, dtype=torch.int32, device="cuda")
         clada.clada_selftest_meeting(ws, n, late, report, status)
         got = report.tolist()
-        if late < 0:
-            assert sorted(got) == [[0, 0]] * (n - 1) + [[0, 1]]
-        elif late in (0, n):
+        if late in (0, n):
             assert got == [[c, n] for c in range(n)]
         else:
             assert [parts for _, parts in got[:n - late]] == [0] * (n - late)
