@@ -136,6 +136,16 @@ int clada_selftest_bounded_waits(void *ws, size_t ws_bytes, uint32_t poll_limit,
 int clada_selftest_meeting(void *ws, size_t ws_bytes, int32_t n_ctas, int32_t n_late, int32_t *report,
                            int32_t *status, void *stream);
 
+/* Self-test of the waits between the CTAs of a batched decode launch (the paper has
+ * no counterpart): four CTAs exchange as a group, one of which begins 5 us x poll_limit
+ * (100 .. 1000) after the others, several times as late as poll_limit polls take.  A
+ * wait that runs out begins anew while a member has not begun, so nobody gives up.
+ *   report      out [4] int32, device: 1 where the wait ended well, 0 where it gave up
+ *               (and status has CLADA_STATUS_TIMEOUT)
+ * The workspace's control words are zero before and after. */
+int clada_selftest_late_member(void *ws, size_t ws_bytes, uint32_t poll_limit, int32_t *report,
+                               int32_t *status, void *stream);
+
 /* out[j] = ||W_out,j||_2 = the l2 norm of row j of w_down_t, fp32.  Once per
  * layer; the second factor of Eq. neuron_activation. */
 int clada_down_norms(const clada_layer *layer, float *out /*[d_ff]*/, void *stream);

@@ -26,7 +26,7 @@ _INT_RETURNING = [
     "clada_workspace_init", "clada_down_norms", "clada_prefix_scores", "clada_refine_scores",
     "clada_select", "clada_prefix_select", "clada_tau_from_sparsity", "clada_cogload",
     "clada_adjust_threshold", "clada_cogload_adjust", "clada_sparse_ffn_decode",
-    "clada_sparse_ffn_decode_static", "clada_sparse_ffn_decode_layers", "clada_selftest_bounded_waits", "clada_selftest_meeting", "clada_cett_threshold_search",
+    "clada_sparse_ffn_decode_static", "clada_sparse_ffn_decode_layers", "clada_selftest_bounded_waits", "clada_selftest_meeting", "clada_selftest_late_member", "clada_cett_threshold_search",
     "clada_cett_curve",
 ]
 
@@ -82,6 +82,7 @@ def load() -> ctypes.CDLL:
     L.clada_workspace_init.argtypes = [vp, sz, vp]
     L.clada_selftest_bounded_waits.argtypes = [vp, sz, ctypes.c_uint32, vp, vp, vp]
     L.clada_selftest_meeting.argtypes = [vp, sz, i32, i32, vp, vp, vp]
+    L.clada_selftest_late_member.argtypes = [vp, sz, ctypes.c_uint32, vp, vp, vp]
     L.clada_down_norms.argtypes = [lp, vp, vp]
     L.clada_prefix_scores.argtypes = [lp, vp, vp, i32, vp, vp, sz, vp, vp]
     L.clada_refine_scores.argtypes = [lp, vp, vp, i32, vp, vp, i32, f32, vp, vp, sz, vp, vp]
@@ -240,6 +241,14 @@ def clada_selftest_meeting(ws, n_ctas: int, n_late: int, report, status=None, st
     _check(load().clada_selftest_meeting(_ptr(ws, torch.uint8, "ws"), ws.numel(), int(n_ctas), int(n_late),
                                          _ptr(report, torch.int32, "report"), _ptr(status, torch.int32, "status"),
                                          _stream(stream)), "clada_selftest_meeting")
+
+
+def clada_selftest_late_member(ws, poll_limit: int, report, status=None, stream=None) -> None:
+    if report.numel() < 4:
+        raise CladaError("report must be [4]")
+    _check(load().clada_selftest_late_member(_ptr(ws, torch.uint8, "ws"), ws.numel(), int(poll_limit),
+                                             _ptr(report, torch.int32, "report"), _ptr(status, torch.int32, "status"),
+                                             _stream(stream)), "clada_selftest_late_member")
 
 
 def clada_down_norms(layer: Layer, out: torch.Tensor, stream=None) -> None:

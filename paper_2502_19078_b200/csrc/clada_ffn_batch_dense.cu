@@ -68,7 +68,6 @@ constexpr int bd_tiles_in_tmem(int seqs) { return (int)kBdTmemCols / (kBdParts *
 constexpr int kBdGroupWord0 = 8;     // group byte counters: control-block words 8..63
 constexpr int kBdMaxGroups = 4 * (64 - kBdGroupWord0);
 constexpr size_t kBdSmemMin = 120 * 1024;
-constexpr unsigned kBdGroupSpinLimit = 1u << 22;
 
 // Opt-in timeline (-DCLADA_BD_TRACE): %globaltimer stamps per CTA, 64 slots, written by the thread that passes the point.
 #ifdef CLADA_BD_TRACE
@@ -250,7 +249,9 @@ sparse_ffn_batch_dense_kernel(const __grid_constant__ CUtensorMap map_x, const _
     pdl_wait();  // x, the scores and the thresholds may come from the launch before
     // CTAs are numbered in the order in which they begin.  The launch is a plain one, so nothing promises that all CTAs
     // are resident at a time; but with these numbers every group but the last one begun is complete whenever a CTA
-    // waits, goes through to the end by itself and makes room for the others.
+    // waits, goes through to the end by itself and makes room for the others.  The last one's three CTAs at most wait, in
+    // group_wait, for a member that other work keeps off the SMs; the waits behind it (of the MMA thread for the others' h,
+    // of the producer for the stages that hold their rows) are as long.
     if (threadIdx.x == 0) s_cta = (int)grid_enter(p.ctrl);
     __syncthreads();
     const int cta = s_cta;
@@ -289,7 +290,7 @@ sparse_ffn_batch_dense_kernel(const __grid_constant__ CUtensorMap map_x, const _
             // first set (their h is here before the group's exchange is over), then tile by tile the other three
             // members' rows; a tile of a later set takes its four members' rows in the same order.
             auto issue_p2 = [&](int mm, int t) -> bool {
-                if (!tc_mbar_wait(tc_smem_u32(&s_empty[s]), par ^ 1, abort_flag)) return false;
+                if (!tc_mbar_wait(tc_smem_u32(&s_empty[s]), par ^ 1, abort_flag, kPlaceLimit)) return false;
                 const int rows0 = (grp * kBdMembers + mm) * p.rows_blk;
                 const uint32_t bar = tc_smem_u32(&s_full[s]);
                 const uint32_t dst = smem0 + (uint32_t)s * stage_bytes;
@@ -389,7 +390,7 @@ sparse_ffn_batch_dense_kernel(const __grid_constant__ CUtensorMap map_x, const _
             tc_fence_after();
             BD_TRACE(3);
             for (int t = 0; t < min(nt, p.tile_set) && ok; ++t) ok = run_p2(dh_own, t, 0u);
-            if (ok && !tc_mbar_wait(tc_smem_u32(&s_h_all), 0, abort_flag)) ok = false;
+            if (ok && !tc_mbar_wait(tc_smem_u32(&s_h_all), 0, abort_flag, kPlaceLimit)) ok = false;
             tc_fence_after();
             for (int t = 0, slot = 0; t < nt && ok; ++t) {
                 if (t >= p.tile_set) {  // the slot's tile of the set before has to be out of the tensor memory
@@ -495,14 +496,7 @@ sparse_ffn_batch_dense_kernel(const __grid_constant__ CUtensorMap map_x, const _
             int gok = 0;
             if (ok && !*abort_flag) {
                 asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(word), "r"(1u << shift) : "memory");
-                for (unsigned spins = 0; spins < kBdGroupSpinLimit; ++spins) {
-                    unsigned seen;
-                    asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(seen) : "l"(word) : "memory");
-                    if (((seen >> shift) & 0xffu) >= (unsigned)kBdMembers) {
-                        gok = 1;
-                        break;
-                    }
-                }
+                gok = group_wait(p.ctrl, word, shift, kBdMembers, (unsigned)(grp + 1) * kBdMembers) ? 1 : 0;
             }
             s_group_ok = gok;
             BD_TRACE(7);

@@ -54,9 +54,44 @@ meeting_selftest_kernel(WsCtrl *ctrl, int n_late, int32_t *report, int32_t *stat
     }
 }
 
+// A group of four CTAs one of which begins delay_ns after the others, longer than poll_limit polls take.
+__global__ void __launch_bounds__(64, 1)
+late_member_selftest_kernel(WsCtrl *ctrl, unsigned poll_limit, unsigned long long delay_ns, int32_t *report, int32_t *status) {
+    unsigned *word = reinterpret_cast<unsigned *>(ctrl) + 8;
+    const unsigned n = gridDim.x, cta = blockIdx.x;
+    if (threadIdx.x == 0) {
+        unsigned long long t0, t;
+        asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t0));
+        t = t0;
+        for (unsigned i = 0; cta == n - 1 && i < kBarrierSpinLimit && t - t0 < delay_ns; ++i) {
+            __nanosleep(1000);
+            asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+        }
+        grid_enter(ctrl);
+        __threadfence();
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(word) : "memory");
+        const bool ok = group_wait(ctrl, word, 0, n, n, poll_limit);
+        report[cta] = ok ? 1 : 0;
+        if (!ok && status) atomicOr(status, CLADA_STATUS_TIMEOUT);
+    }
+    const GridPart mine = grid_meet(ctrl, n, (int)cta, 32);
+    if (threadIdx.x == 0 && mine.parts > 0 && mine.part == 0) *word = 0u;
+}
+
 }  // namespace clada
 
 using namespace clada;
+
+extern "C" int clada_selftest_late_member(void *ws, size_t ws_bytes, uint32_t poll_limit, int32_t *report, int32_t *status,
+                                          void *stream) {
+    if (!ws || !report) return CLADA_ERR_NULL;
+    if (ws_bytes < kWsCtrlBytes || (reinterpret_cast<uintptr_t>(ws) & 255u)) return CLADA_ERR_WORKSPACE;
+    if (poll_limit < 100 || poll_limit > 1000) return CLADA_ERR_SHAPE;
+    late_member_selftest_kernel<<<4, 64, 0, static_cast<cudaStream_t>(stream)>>>(static_cast<WsCtrl *>(ws), poll_limit, 5000ull * poll_limit,
+                                                                              report, status);
+    CLADA_CUDA_TRY(cudaGetLastError());
+    return CLADA_OK;
+}
 
 extern "C" int clada_selftest_meeting(void *ws, size_t ws_bytes, int32_t n_ctas, int32_t n_late, int32_t *report,
                                       int32_t *status, void *stream) {

@@ -119,6 +119,29 @@ static __device__ GridPart grid_meet(WsCtrl *ctrl, unsigned n_ctas, int cta, int
     return mine;
 }
 
+// Members of a group of CTAs of one launch wait for one another: byte `shift` of *word counts those that are ready, `need`
+// CTAs of the launch have begun when all members have.  Nothing promises when the scheduler places a member that has not
+// begun: other work may hold the SMs that it needs.  So a wait that has run out begins anew, kPlaceRounds times (about a
+// minute), while a member has not begun, and once more when all have.
+constexpr unsigned kGroupSpinLimit = 1u << 22, kPlaceRounds = 32;
+constexpr unsigned kPlaceLimit = 1u << 26;  // tries of at most ~1 us: mbarrier waits behind such a wait
+static __device__ bool group_wait(const WsCtrl *ctrl, const unsigned *word, unsigned shift, unsigned members, unsigned need,
+                                  unsigned spin_limit = kGroupSpinLimit) {
+    unsigned spins = 0, rounds = 0;
+    bool begun = false;
+    for (;;) {
+        unsigned seen;
+        asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(seen) : "l"(word) : "memory");
+        if (((seen >> shift) & 0xffu) >= members) return true;
+        if (++spins <= spin_limit) continue;
+        if (begun || ++rounds > kPlaceRounds) return false;
+        unsigned long long now;
+        asm volatile("ld.relaxed.gpu.u64 %0, [%1];" : "=l"(now) : "l"(ctrl) : "memory");
+        begun = (unsigned)(now >> 32) >= need;
+        spins = 0;
+    }
+}
+
 // ---- mbarrier / bulk-copy primitives (bounded waits) -------------------------------------------
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {

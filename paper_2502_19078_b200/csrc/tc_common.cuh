@@ -27,8 +27,9 @@ __device__ __forceinline__ void tc_mbar_expect_tx(uint32_t bar, uint32_t bytes) 
 }
 // Bounded wait for the phase of the given parity; false if it gave up or another role raised the
 // abort flag.  Each try suspends for at most ~1 us (the hint), so the bound is about a second.
-__device__ __forceinline__ bool tc_mbar_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag) {
-    for (unsigned i = 0; i < kTcSpinLimit; ++i) {
+__device__ __forceinline__ bool tc_mbar_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag,
+                                             unsigned limit = kTcSpinLimit) {
+    for (unsigned i = 0; i < limit; ++i) {
         uint32_t ok;
         asm volatile(
             "{\n\t.reg .pred p;\n\t"

@@ -134,3 +134,12 @@ def test_parts_of_a_meeting(clada, n, late):
             assert [parts for _, parts in got[:n - late]] == [0] * (n - late)
             assert sorted(got[n - late:]) == [[c, late] for c in range(late)]
         assert int(status.item()) == 0 and int(ws.view(torch.int32).abs().sum().item()) == 0
+
+
+@pytest.mark.parametrize("limit", [100, 1000])
+def test_a_group_waits_for_a_member_that_begins_late(clada, limit):
+    ws = torch.zeros(256, dtype=torch.uint8, device="cuda")
+    status, report = torch.zeros(1, dtype=torch.int32, device="cuda"), torch.full((4,), -9, dtype=torch.int32, device="cuda")
+    clada.clada_selftest_late_member(ws, limit, report, status)
+    assert report.tolist() == [1, 1, 1, 1]
+    assert int(status.item()) == 0 and int(ws.view(torch.int32).abs().sum().item()) == 0
