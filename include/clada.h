@@ -109,14 +109,14 @@ int clada_stream_read_probe(const void *buf, size_t bytes, uint32_t *sink, void 
 
 /* Self-test of the bounded device-side waits (the paper has no counterpart).
  * Every wait inside the decode kernels -- for a ring stage's mbarrier, for the
- * grid barrier -- gives up after a bounded number of polls and reports
- * CLADA_STATUS_TIMEOUT instead of hanging.  This call makes both kinds of wait
- * run out on purpose, in a form that cannot hang: two small CTAs wait on a
- * shared-memory barrier that nobody arrives at, then meet at the workspace's
- * grid barrier, which is told to expect one CTA more than the grid has.
+ * other CTAs of the launch -- gives up after a bounded number of polls and reports
+ * CLADA_STATUS_TIMEOUT instead of hanging.  This call makes an mbarrier wait and
+ * the launch's meeting run out on purpose, in a form that cannot hang: two small
+ * CTAs wait on a shared-memory barrier that nobody arrives at, then come to a
+ * meeting of three, the third of which is counted as begun and never comes.
  *   poll_limit  polls per wait before giving up, 1 .. 2^20 (a few thousand is plenty)
  *   report      out [2] int32, device: report[0] = 1 if the mbarrier wait gave up,
- *               report[1] = 1 if the grid barrier gave up (both are expected)
+ *               report[1] = 1 if the meeting gave up (both are expected)
  *   status      optional device word; CLADA_STATUS_TIMEOUT is or-ed into it
  * Afterwards the workspace's control words are left as a timed-out decode
  * kernel leaves them (non-zero): call clada_workspace_init before the next

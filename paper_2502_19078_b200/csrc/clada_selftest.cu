@@ -1,6 +1,6 @@
-// Self-test of the bounded waits: the decode kernels' two wait primitives (an mbarrier wait and the grid
-// barrier) are made to run out in a harmless form -- a barrier nobody arrives at, a grid barrier that
-// expects one CTA more than the grid has -- with a small poll limit, so that the give-up branch, the
+// Self-test of the bounded waits: the decode kernels' two wait primitives (an mbarrier wait and the grid's
+// meeting) are made to run out in a harmless form -- a barrier nobody arrives at, a meeting to which one CTA
+// that is counted as begun never comes -- with a small poll limit, so that the give-up branch, the
 // status bit and the recovery by clada_workspace_init can be exercised without any kernel ever hanging.
 #include "common.cuh"
 #include "ffn_common.cuh"
@@ -21,13 +21,21 @@ bounded_wait_selftest_kernel(WsCtrl *ctrl, unsigned poll_limit, int32_t *report,
     if (!mbar_wait(smem_u32(&bar), 0, poll_limit)) atomicOr(&gave_up, 1);
     __syncthreads();
     const bool mbar_gave_up = gave_up != 0;
-    // the grid barrier of a grid of gridDim.x CTAs that is told to expect one more
-    const bool barrier_ok = grid_barrier(ctrl, gridDim.x + 1u, 32, poll_limit);
+    // the meeting of one CTA more than the grid has, all of them counted as begun
+    const unsigned n = gridDim.x + 1u;
+    if (threadIdx.x == 0) {
+        grid_enter(ctrl);
+        if (blockIdx.x == 0) grid_enter(ctrl);
+        unsigned begun = 0;
+        for (unsigned i = 0; i < kBarrierSpinLimit && begun < n; ++i)
+            asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(begun) : "l"(&ctrl->started) : "memory");
+    }
+    const bool meeting_ok = grid_meet(ctrl, n, (int)blockIdx.x, 32, poll_limit).parts >= 0;
     if (threadIdx.x == 0 && blockIdx.x == 0) {
         report[0] = mbar_gave_up ? 1 : 0;
-        report[1] = barrier_ok ? 0 : 1;
+        report[1] = meeting_ok ? 0 : 1;
     }
-    if (threadIdx.x == 0 && (mbar_gave_up || !barrier_ok) && status) atomicOr(status, CLADA_STATUS_TIMEOUT);
+    if (threadIdx.x == 0 && (mbar_gave_up || !meeting_ok) && status) atomicOr(status, CLADA_STATUS_TIMEOUT);
 }
 
 // The meeting with CTAs that begin late, as where other work holds SMs: of n CTAs the last n_late begin only after the others

@@ -1,5 +1,5 @@
 // Device primitives shared by the single-sequence and the batched sparse-FFN decode kernels:
-// bounded grid barrier, bounded mbarrier waits, bulk row copies with L2 policies, packed-pair unpacking.
+// the bounded meeting of a launch's CTAs, bounded mbarrier waits, bulk row copies with L2 policies, packed-pair unpacking.
 #pragma once
 
 #include "common.cuh"
@@ -7,42 +7,6 @@
 namespace clada {
 
 constexpr unsigned kBarrierSpinLimit = 1u << 22;  // polls of an L2 word: gives up after ~1 s at most
-
-// Bounded grid-wide barrier on two self-resetting counters in the workspace control block.
-// Returns false if the wait expired.  Thread 0 arrives and polls; the departure count (whose last
-// increment resets both counters for the next launch) is another round trip to L2 that nothing waits
-// for, so a thread of the otherwise idle producer warp takes it after the CTA has been released.
-static __device__ bool grid_barrier(WsCtrl *ctrl, unsigned n_ctas, int depart_tid,
-                                    unsigned spin_limit = kBarrierSpinLimit) {
-    __shared__ int s_ok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(&ctrl->arrive, 1u);
-        unsigned spins = 0, seen;
-        int ok = 1;
-        for (;;) {
-            asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(seen) : "l"(&ctrl->arrive) : "memory");
-            if (seen >= n_ctas) break;
-            if (++spins > spin_limit) {
-                ok = 0;
-                break;
-            }
-        }
-        s_ok = ok;
-    }
-    __syncthreads();
-    const bool ok = s_ok != 0;
-    if ((int)threadIdx.x == depart_tid && ok) {
-        const unsigned left = atomicAdd(&ctrl->depart, 1u);
-        if (left == n_ctas - 1) {  // last one out: everyone has seen arrive == n_ctas
-            ctrl->arrive = 0;
-            ctrl->depart = 0;
-            __threadfence();
-        }
-    }
-    return ok;
-}
 
 // Grid-wide meeting of a plain launch, whose CTAs need not all be resident at once.  A cooperative launch begins only
 // after its predecessor has left the SMs; a plain one has its CTAs in place (barriers set up, in griddepcontrol.wait)
@@ -76,6 +40,8 @@ struct GridPart {
     int part, parts;
 };
 constexpr unsigned kMeetCount = 0xffffu, kMeetLeft = 0x10000u;  // arrive: CTAs that came; one that left at once
+// Thread 0 comes and polls; the departure, whose last one clears the control words, is another round trip to L2 that nothing
+// waits for, so an otherwise idle thread (depart_tid) takes it.  A wait that gave up leaves the words as they are.
 // cta: this CTA's part when all wait.  The way of a launch that is alone on the device is an addition and a poll, as in a
 // plain barrier (a second fence behind the poll and the added word's return trip before it made FFN launches in a graph 8.8
 // us instead of 8.4 on 512 x 1376 fp32, 13.3 instead of 12.8 on 1024 x 4100, 34.6 instead of 34.4 on 4096 x 11008).

@@ -1,5 +1,5 @@
 """The bounded device-side waits, made to run out in the harmless form: clada_selftest_bounded_waits waits on a
-shared-memory barrier nobody arrives at and on a grid barrier told to expect one CTA too many, with a small poll
+shared-memory barrier nobody arrives at and comes to a meeting of one CTA too many, with a small poll
 limit.  The kernel must return, report both give-ups and raise CLADA_STATUS_TIMEOUT; the workspace's control
 words are then dirty, and after clada_workspace_init ordinary decodes on the same workspace (per-layer launch,
 tile of sequences, persistent stack launch) match the oracle again.  Nothing here faults, traps or waits
@@ -84,3 +84,31 @@ def test_selftest_refuses_bad_arguments(clada):
     with pytest.raises(clada.CladaError):
         clada.clada_selftest_bounded_waits(ws[:64], 100, report)      # no room for the control words
     torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("B,dtype", [(1, torch.bfloat16), (2, torch.bfloat16), (2, torch.float32), (6, torch.bfloat16)])
+def test_every_kind_of_launch_that_meets_recovers(clada, B, dtype):
+    """One sequence, tiles of two on both kinds of cores, the dense pass: the meeting's give-up leaves both CTAs that came
+    and all three that began in the control words, and after clada_workspace_init the launch's bits are those of before."""
+    g = torch.Generator(device="cuda").manual_seed(7)
+    mk = lambda *s: torch.randn(s, generator=g, device="cuda").mul_(0.05).to(dtype)
+    layer, x = clada.Layer(mk(900, 512), mk(900, 512), mk(900, 512)), mk(B, 512)
+    scores, tau = torch.rand(B, 900, generator=g, device="cuda"), torch.full((B,), 0.4, device="cuda")
+    ws = clada.new_workspace(layer, B, 0)
+    report = torch.zeros(2, dtype=torch.int32, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+
+    def decode():
+        y = torch.full((B, 512), float("nan"), device="cuda")
+        clada.clada_sparse_ffn_decode(layer, x, scores, tau, 1, y, ws, status=status)
+        return y
+
+    want = decode()
+    assert int(status.item()) == 0
+    clada.clada_selftest_bounded_waits(ws, 100, report, status)
+    assert report.tolist() == [1, 1] and int(status.item()) == clada.STATUS_TIMEOUT
+    assert ws[:16].view(torch.int32).tolist() == [2, 3, 0, 0]
+    clada.clada_workspace_init(ws)
+    status.zero_()
+    assert torch.equal(decode(), want) and int(status.item()) == 0
+    assert int(ws[:256].view(torch.int32).abs().sum().item()) == 0
