@@ -20,7 +20,7 @@
 // Measured (us a step with its cognitive load, a launch per sequence / this way): four of 2048 x 16384, a vocabulary of
 // 256000, 96.3 / 68.6; three, four and eight of 2048 x 16384 78.3 / 64.7, 103 / 73.5, 201 / 121; of 4096 x 11008 92.7 / 84.5,
 // 121 / 99, 236 / 183; of 5120 x 13824 133 / 123, 176 / 143, 346 / 287; of 1024 x 4100 41.2 / 31.4, 53.8 / 33.3, 103 / 45.9.
-// Two sequences keep a launch each: 26.7 / 26.6, 51.5 / 52.6, 59.8 / 68.7 and 88.5 / 96.9 on these layers.
+// Which batches do: at nb_plan.
 #include <algorithm>
 
 #include "common.cuh"
@@ -535,14 +535,24 @@ struct NbPlan {
     size_t smem_hidden, smem_down, smem_keep;
 };
 
+// Which batches take a pass; measured against a launch per sequence, both in graphs, layers of 4096 to 24576 neurons, lists of
+// independent random neurons, of ones half shared, of the same ones and of none in common (times a pass / its launches):
+//   four and more  0.55 to 0.98 up to 6144 columns (lists without a neuron in common up to 1.10), while the ring has five stages
+//                  beside x; with four 1.1 to 1.2 (7168 gated columns from six sequences on, 8192 from four)
+//   three          0.80 to 1.0 on rows of up to 256 vectors and of 512 and more, with six stages (with five, 8192 gated columns,
+//                  1.04 to 1.06); on rows of 257 to 511 a single launch is at its best: layers without a gate 1.03 to 1.14, gated ones
+//                  0.94 to 1.0 up to 80 MB a matrix (2304 x 16384, 3072 x 12288), 1.01 to 1.06 beyond
+//   two            steps of 1024 x 4100 26.7 / 26.6 us, 2048 x 16384 51.5 / 52.6, 4096 x 11008 59.8 / 68.7, 5120 x 13824 88.5 / 96.9
 static bool nb_plan(const clada_layer *L, int nb, const DeviceInfo &di, NbPlan *pl) {
     const int vpr = nb_vpr(L);
-    if (nb < 1 || nb > kNestedBatchMax || vpr > 2 * kConsumers || L->d_ff > kSingleMaxDff) return false;
-    const size_t row = (size_t)vpr * 16, stage = (act_is_gated(L->activation) ? 2 : 1) * row;
+    const bool gated = act_is_gated(L->activation);
+    if (nb < kNestedBatchMin || nb > kNestedBatchMax || vpr > 2 * kConsumers || L->d_ff > kSingleMaxDff) return false;
+    const size_t row = (size_t)vpr * 16, stage = (gated ? 2 : 1) * row;
+    if (nb == 3 && vpr > kConsumers / 2 && vpr < kConsumers && (!gated || row * L->d_ff > ((size_t)80 << 20))) return false;
     const size_t cap = (size_t)(L->d_ff / di.num_sms + 2);
     const size_t tail = (size_t)nb * row + 2 * kNbMaxStages * sizeof(uint64_t) + 2 * cap * sizeof(int);
     const size_t budget = (size_t)di.max_smem_optin - kNbStatic;
-    if (budget < tail + 4 * stage) return false;
+    if (budget < tail + (nb == 3 ? 6 : 5) * stage) return false;
     const int fit = (int)std::min<size_t>(kNbMaxStages, (budget - tail) / stage);
     pl->n_cons = std::min(fit - std::max(2, fit / 3), kNbConsWarps);  // the other stages are on their way
     pl->n_stages = fit;

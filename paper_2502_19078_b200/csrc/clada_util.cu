@@ -150,8 +150,12 @@ size_t clada_workspace_bytes(const clada_layer *layer, int32_t B, int64_t T_tota
         // sequences past a multiple of 32 may still run as tiles, whose keep words sit behind the launch scratch
         decode = std::max(decode, dense + ((((size_t)B * ((size_t)(layer->d_ff + 31) / 32) * sizeof(unsigned)) + 255) & ~(size_t)255));
     }
-    // several sequences over nested lists in one pass
-    if (B >= kNestedBatchMin) decode = std::max(decode, nested_batch_scratch_bytes(layer, std::min(B, kNestedBatchMax), sms));
+    // several sequences over nested lists in one pass, the most that take one
+    for (int nb = std::min(B, kNestedBatchMax); nb >= kNestedBatchMin; --nb) {
+        if (!nested_batch_supported(layer, nb)) continue;
+        decode = std::max(decode, nested_batch_scratch_bytes(layer, nb, sms));
+        break;
+    }
     // prefix: one fp32 partial sum of squares per (token tile, neuron); tiles hold 64 tokens
     size_t tiles = (size_t)(T_total / 64) + (size_t)B + 1;
     size_t prefix = (tiles * (size_t)layer->d_ff * sizeof(float) + 255) & ~(size_t)255;

@@ -7,8 +7,9 @@
 namespace clada {
 
 constexpr int kNestedBatchMax = 8;  // sequences of one pass
-constexpr int kNestedBatchMin = 3;  // fewer have a launch each (measured in clada_nested_batch.cu)
+constexpr int kNestedBatchMin = 3;  // fewer have a launch each
 
+// Whether nb sequences of this layer take a pass (the measurements behind it are at nb_plan).
 bool nested_batch_supported(const clada_layer *layer, int nb);
 // Scratch of a pass behind the control block: hidden values, keep words, partial rows.
 size_t nested_batch_scratch_bytes(const clada_layer *layer, int nb, int num_sms);

@@ -79,3 +79,27 @@ def test_launches_do_not_grow_with_the_batch(clada):
     ws, y = clada.new_workspace(layer, 8, 0), torch.empty(8, 512, device="cuda")
     names = [n for n, _ in launches(lambda: clada.clada_sparse_ffn_decode_nested(layer, x, order, counts, level, y, ws))]
     assert len(names) == 4 and not any("sparse_ffn_kernel" in n for n in names), names
+
+
+@pytest.mark.parametrize("B,d,F,dtype,act,singles,passes", [
+    (2, 1024, 300, torch.bfloat16, 0, 2, 0),                                            # two: a launch each
+    (3, 2048, 300, torch.float16, 2, 0, 1), (3, 2056, 300, torch.float16, 2, 3, 0),     # three, no gate: rows of 256, 257,
+    (3, 4088, 300, torch.float16, 2, 3, 0), (3, 4096, 300, torch.float16, 2, 0, 1),     # 511 and 512 vectors
+    (3, 2560, 16384, torch.bfloat16, 0, 0, 1), (3, 2560, 16385, torch.bfloat16, 0, 3, 0),  # gated: 80 MB a matrix
+    (3, 7168, 300, torch.bfloat16, 0, 0, 1), (3, 7680, 300, torch.bfloat16, 0, 3, 0),   # six ring stages beside x, and five
+    (5, 7168, 300, torch.bfloat16, 0, 0, 1), (6, 7168, 300, torch.bfloat16, 0, 1, 1),   # five, and four: a pass of five
+    (4, 8192, 300, torch.bfloat16, 0, 4, 0), (8, 8192, 300, torch.float16, 2, 0, 1),
+    (4, 2560, 300, torch.float32, 0, 0, 1), (4, 4096, 300, torch.float32, 1, 4, 0),
+    (11, 512, 300, torch.bfloat16, 1, 0, 2), (17, 512, 300, torch.float32, 0, 1, 2),
+])
+def test_which_batches_take_a_pass(clada, B, d, F, dtype, act, singles, passes):
+    """Both sides of each line of the rule, and the same bits from a launch per sequence."""
+    layer, order, counts, level, x = _case(clada, B, d, F, dtype, act)
+    ws, y = clada.new_workspace(layer, B, 0), torch.empty(B, d, device="cuda")
+    names = [n for n, _ in launches(lambda: clada.clada_sparse_ffn_decode_nested(layer, x, order, counts, level, y, ws))]
+    assert sum("sparse_ffn_kernel" in n for n in names) == singles and sum("nested_sums_kernel" in n for n in names) == passes
+    assert len(names) == singles + 4 * passes
+    y = _run(clada, layer, order, counts, level, x, torch.float32, ws)
+    for b in range(B):
+        s = slice(b, b + 1)
+        assert torch.equal(y[s], _run(clada, layer, order[s], counts[s], level[s], x[s], torch.float32, ws)), b
