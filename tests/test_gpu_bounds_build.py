@@ -1,6 +1,6 @@
 """The index-checking build (-DCLADA_DEBUG_BOUNDS): every neuron index is range-checked on its way into a row
 address or a list slot, a bad one raises CLADA_STATUS_BAD_INDEX in the call's status word and is made harmless.
-Parity cases of the decode calls (one sequence, the stack launch, tiles, nested lists, and the dense pass, which
+Parity cases of the decode calls (one sequence, the stack launch, tiles, nested lists alone and in shared passes, and the dense pass, which
 gathers nothing) run on that build in a child process: they pass against the oracle as on the release build, and the status words they
 assert on stay 0 -- no check fires on any list the kernels build themselves.
 """
@@ -24,6 +24,7 @@ CASES = [
     "tests/test_gpu_batch_dense.py::test_stack_call_with_a_batch_runs_dense_passes",
     "tests/test_gpu_stack.py",
     "tests/test_gpu_nested.py",
+    "tests/test_gpu_nested_batch.py::test_batch_bits_are_those_of_single_launches",
 ]
 
 

@@ -1,6 +1,8 @@
 """Decode launches whose CTAs cannot all be resident at a time: beside a kernel that keeps half of the SMs for longer than
 a decode takes, and beside another decode on a second stream.  Every launch ends, its control words are back at zero and
-its outputs are the bits of an undisturbed run."""
+its outputs are the bits of an undisturbed run.  (Five sequences over lists take passes that do not meet; they are there
+for their chained launches.)  How far two kernels overlap is the scheduler's affair, so who leaves a meeting, who shares the
+parts and how a group waits for a late member is checked in self-tests whose CTAs are made to begin late."""
 import pytest
 import torch
 

@@ -1,6 +1,7 @@
 """Nested decode of several sequences in shared passes: every sequence gets the bits of a launch of its own, at the edges
 of its tiles (rows of one vector, of one or two consumer groups, of two vectors per thread; layers smaller than the grid;
-empty, whole and one-neuron lists; passes of two to eight sequences and rests), with any workspace that was accepted."""
+empty, whole and one-neuron lists; passes of three to eight sequences and rests, two sequences in a launch each), with any
+workspace that was accepted, with inputs out of range, and from a graph whose launches wait for one another."""
 import pytest
 import torch
 
@@ -49,6 +50,8 @@ def _run(clada, layer, order, counts, level, x, y_dtype, ws):
     (8, 5120, 450, torch.bfloat16, 0), (3, 8192, 300, torch.bfloat16, 0), (6, 8192, 300, torch.float16, 2),
     (3, 512, 1376, torch.float32, 0), (4, 1024, 640, torch.float32, 2), (8, 1032, 640, torch.float32, 1),
     (3, 4096, 200, torch.float32, 0), (10, 256, 40000, torch.bfloat16, 0),
+    (3, 8, 1, torch.bfloat16, 0), (3, 1024, 13400, torch.bfloat16, 2), (4, 4104, 700, torch.float16, 0),
+    (4, 8192, 300, torch.bfloat16, 2), (4, 2568, 200, torch.float32, 0),
 ])
 def test_batch_bits_are_those_of_single_launches(clada, B, d, F, dtype, act):
     layer, order, counts, level, x = _case(clada, B, d, F, dtype, act)
@@ -103,3 +106,82 @@ def test_which_batches_take_a_pass(clada, B, d, F, dtype, act, singles, passes):
     for b in range(B):
         s = slice(b, b + 1)
         assert torch.equal(y[s], _run(clada, layer, order[s], counts[s], level[s], x[s], torch.float32, ws)), b
+
+
+@pytest.mark.parametrize("d,dtype", [(512, torch.bfloat16), (1032, torch.float32)])
+@pytest.mark.parametrize("B,bad", [(3, 0), (3, 2), (8, 7)])
+@pytest.mark.parametrize("kind", ["level below", "level above", "count below", "count above", "indices"])
+def test_inputs_out_of_range_are_clamped_and_reported(clada, B, bad, d, dtype, kind):
+    """One sequence's level, count or indices outside the layer: reported, made harmless as a launch of its own makes them,
+    and nothing to the other sequences."""
+    F = 700
+    layer, order, counts, level, x = _case(clada, B, d, F, dtype, 0)
+    counts[bad] = torch.tensor([60, 300, 100, 200])
+    clean = _run(clada, layer, order, counts, level, x, torch.float32, clada.new_workspace(layer, B, 0))
+    if kind.startswith("level"):
+        level[bad] = -1 if kind == "level below" else 6
+    elif kind.startswith("count"):
+        counts[bad] = -3 if kind == "count below" else F + 5
+    else:
+        order[bad, :60:7] = torch.tensor([-7, F, F + 100, -2 ** 31, 2 ** 31 - 1, -1, F, F, 2 * F], dtype=torch.int32, device="cuda")
+
+    def run(s, ws):
+        y, kept = torch.full((B, d), 7.0, device="cuda")[s], torch.full((B,), -1, dtype=torch.int32, device="cuda")[s]
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        clada.clada_sparse_ffn_decode_nested(layer, x[s], order[s], counts[s], level[s], y, ws, kept, status)
+        return y, kept, int(status.item())
+
+    y, kept, status = run(slice(0, B), clada.new_workspace(layer, B, 0))
+    assert status == 8  # CLADA_STATUS_BAD_INDEX
+    one = clada.new_workspace(layer, 1, 0)
+    for b in range(B):
+        yb, kb, sb = run(slice(b, b + 1), one)
+        assert torch.equal(y[b:b + 1], yb) and torch.equal(kept[b:b + 1], kb) and (sb != 0) == (b == bad)
+        if b != bad:
+            assert torch.equal(y[b], clean[b])
+
+
+@pytest.mark.parametrize("B,d,F,dtype", [(4, 2048, 1500, torch.bfloat16), (3, 1024, 4100, torch.float16), (9, 512, 700, torch.bfloat16)])
+def test_a_graph_that_feeds_each_launch_from_the_one_before(clada, B, d, F, dtype):
+    """Two of a pass's launches read ahead of their wait: in a graph that makes the lists, decodes over them and decodes
+    again from that output, replayed with other inputs each time, every read comes after what writes it."""
+    layer, order, counts, _, x = _case(clada, B, d, F, dtype, 1)
+    ws, status = clada.new_workspace(layer, B, 0), torch.zeros(1, dtype=torch.int32, device="cuda")
+    scores, tau = torch.empty(B, F, device="cuda"), torch.full((B,), 0.75, device="cuda")
+    logits, token = torch.empty(B, 3000, device="cuda"), torch.arange(B, dtype=torch.int32, device="cuda")
+    level = torch.zeros(B, dtype=torch.int32, device="cuda")
+    s, h = torch.empty(B, device="cuda"), torch.empty(B, device="cuda")
+    y, z = torch.empty(B, d, dtype=dtype, device="cuda"), torch.empty(B, d, device="cuda")
+
+    def step(sync):
+        for part in (lambda: clada.clada_nested_build(scores, tau, 0.4, 0.2, order, counts),
+                     lambda: clada.clada_cogload_level(logits, token, 8.0, 7.4, s, h, level),
+                     lambda: clada.clada_sparse_ffn_decode_nested(layer, x, order, counts, level, y, ws, None, status),
+                     lambda: clada.clada_sparse_ffn_decode_nested(layer, y, order, counts, level, z, ws, None, status)):
+            part()
+            if sync:
+                torch.cuda.synchronize()
+
+    g = torch.Generator(device="cuda").manual_seed(5)
+
+    def inputs():
+        scores.uniform_(0.5, 1.5, generator=g)
+        logits.normal_(0.0, 3.0, generator=g)
+        x.normal_(0.0, 1.0, generator=g)
+
+    inputs()
+    step(True)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        step(False)
+    for _ in range(20):
+        inputs()
+        torch.cuda.synchronize()
+        graph.replay()
+        torch.cuda.synchronize()
+        got = y.clone(), z.clone(), order.clone(), level.clone()
+        step(True)
+        for a, b in zip(got, (y, z, order, level)):
+            assert torch.equal(a, b)
+        assert torch.isfinite(z).all() and z.abs().max() > 0
+    assert int(status.item()) == 0
