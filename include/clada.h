@@ -93,6 +93,10 @@ const char *clada_last_cuda_error(void);
 
 /* Bytes of workspace that suffice for any call on this layer with B
  * sequences and T_total prefix tokens in all (T_total = 0 for decode-only use).
+ * From three sequences on that holds the shared passes over nested lists, about
+ * a d_model row of 4-byte partial sums per SM and sequence (up to eight; two rows where
+ * d_model takes at most 256 16-byte vectors): 19 MB for eight of 2048 columns.  Nested
+ * calls take less, too, and run as smaller launches then.
  * 0 on invalid arguments. */
 size_t clada_workspace_bytes(const clada_layer *layer, int32_t B, int64_t T_total);
 
@@ -424,8 +428,9 @@ int clada_prefill_down(const clada_layer *layer, const void *w_down, const void 
  * clada_sparse_ffn_decode_nested, per decode step and layer: the sparse FFN over
  * order[b][0 .. counts[b][level[b]]).  Same x / y / workspace / status rules as
  * clada_sparse_ffn_decode (workspace of clada_workspace_bytes(layer, 1, 0) is
- * enough: sequences then run one launch each; with that of the batch three to
- * eight of them share their reads, each with the same bits).  The sum over the kept neurons runs
+ * enough; with that of the batch three to eight sequences share their reads where
+ * that is faster than a launch each, which depends on the layer's shape; a sequence's
+ * bits do not depend on it).  The sum over the kept neurons runs
  * in list order split over the CTAs, so y agrees with clada_sparse_ffn_decode to
  * rounding (fp32 sums in another order), not bit for bit.  count_out [B] or
  * NULL receives the kept count.  A level outside 0..3, a count outside

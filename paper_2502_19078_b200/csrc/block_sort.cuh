@@ -26,7 +26,7 @@ constexpr size_t kSortSmem = (size_t)kSortMaxN * 8 + (size_t)(kSortBuckets + 1) 
 // counting alone.  Bound by latency, memory's first and shared memory's afterwards.  The order inside a piece's slots is
 // arrival order; the ranks do not depend on it.  Measured: lists of 8 sequences of 14336 neurons take 194.5 us a call with
 // the network, 12.5 with every element's piece looked up and the counters scanned one by one (a warp's in four banks), 11.5
-// now; 32 of them 14.0 / 12.5, 16 of 16384 13.7 / 12.2.
+// now; 32 of them 14.0 / 12.5, 16 of 16384 13.7 / 12.2 (back-to-back calls; on scores not seen before half of the gain).
 template <typename Load, typename KeyOf, typename Emit>
 __device__ void block_sort(int n, unsigned reg_lo, unsigned reg_hi, int r0, int r1, unsigned char *smem, Load load,
                            KeyOf key_of, Emit emit) {

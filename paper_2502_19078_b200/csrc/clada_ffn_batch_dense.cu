@@ -25,7 +25,7 @@
 // of a thread in flight together, rows of absent sequences left out) and the final sums (equal runs for every CTA,
 // nineteen loads in flight) are kept short.  A call measured, as two launches or one of 16 columns at first / now: 32
 // sequences of a 13B layer 153.7 / 80.3 us, 16 of it 77.2 / 74.9, 6 of 4096 x 14336 67.9 / 64.8, 6 of 5120 x 4100 62.6 /
-// 61.0, 24 of 1024 x 4100 46.2 / 24.0 (whole steps, with cognitive load: 8 of 4096 x 14336 73.4, 32 of the 13B layer 98.6).
+// 61.0, 24 of 1024 x 4100 46.2 / 24.0 (whole steps, with cognitive load: 8 of 4096 x 14336 69.5, 32 of the 13B layer 95.4).
 // Asking phase 2's boxes into L2 meanwhile (cp.async.bulk.prefetch.tensor, 8 to 48 stages) cost
 // 2.5 to 8 us: the requests are paid for twice.
 //

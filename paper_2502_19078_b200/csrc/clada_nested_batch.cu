@@ -11,7 +11,7 @@
 //   nested_hidden_kernel  the union of the heads shared out evenly; a producer warp streams gate | up rows through a ring
 //                         of stages with bulk copies, a lane per row; a free consumer warp takes the next neuron (no
 //                         CTA-wide step at all), up to four of its sequences at a time, x from shared memory.  Bound by the
-//                         consumers' instructions (0.45 a cycle and scheduler, half of the HBM rate).
+//                         consumers' instructions (0.5 a cycle and scheduler, half of the HBM rate).
 //   nested_down_kernel    CTA c adds up, list after list, the down rows of the share that CTA c of a single launch takes;
 //                         its rows are on their way before the hidden values are waited for.  Bound by HBM and L2 (5 to
 //                         6 TB/s with a third of the rows from L2).

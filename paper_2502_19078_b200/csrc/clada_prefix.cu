@@ -315,7 +315,7 @@ prefix_finalize_kernel(const float *__restrict__ partials, const SeqTable tab, i
 // Chunked prefill: the same tile sums added into a running sum of squares per (prompt, neuron) ...
 // Latency-bound: with one load after the other 7.1 us for the 16 tiles of 2000 tokens (14336 neurons); its launch, the
 // finishing one and the down projection's are chained to what runs before them.  A chunk of 256 tokens (4096 x 11008), three
-// calls, 109 us before and 102.6 now, of 2000 tokens (4096 x 14336) 609 / 604.
+// calls, 109 us before and 102.6 now; of 2000 tokens (4096 x 14336) 627 and 624, which is within what runs differ by.
 __global__ void prefix_accumulate_kernel(const float *__restrict__ partials, const SeqTable tab, int tile, int d_ff,
                                          float *__restrict__ sumsq) {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;

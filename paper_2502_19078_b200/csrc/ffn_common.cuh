@@ -17,9 +17,12 @@ constexpr unsigned kBarrierSpinLimit = 1u << 22;  // polls of an L2 word: gives 
 // beside prompts of 96 tokens on another (112 CTAs each), us a decode and a prompt, cooperative / all parts by the last CTA /
 // shared: one sequence of 4096 x 11008 60 + 87, 81 + 121, 47 + 87; two of 2560 x 10240 61 + 85, 121 + 156, 49 + 85; four of
 // 1024 x 4096 fp32 53 + 79, 92 + 127, 44 + 79; 8 of 4096 x 14336 90 + 117, 113 + 139, 89 + 116; 32 of 5120 x 13824 110 + 136,
-// 101 + 136, 101 + 137.
-// Measured (us a decode step, cooperative / plain): 512 x 1376 fp32 14.8 / 13.9, 1024 x 4100 19.8 / 18.2, 4096 x 11008 39.8 /
-// 38.3, two sequences of 2560 x 10240 31.2 / 29.8, 8 of 4096 x 14336 71.8 / 69.4, 32 of 5120 x 13824 93.2 / 92.0.
+// 101 + 136, 101 + 137.  (Not for all: one of 4096 x 11008 beside prompts of 146 CTAs 89 + 144, then 136 + 137; 32 of 5120 x 13824 beside prompts of 37
+// CTAs 115 + 147, 124 + 157.)
+// What a plain launch gives is the launch latency of calls that follow one another (us a decode step, cooperative / plain):
+// back to back 512 x 1376 fp32 14.7 / 13.1, 1024 x 4100 19.8 / 17.7, 4096 x 11008 41.7 / 39.8, two sequences of 2560 x 10240 37.3 /
+// 35.3, 8 of 4096 x 14336 74.0 / 71.7, 32 of 5120 x 13824 92.2 / 89.5; replayed from a graph, where the cooperative launch
+// waits for little, 12.5 / 12.4, 16.9 / 16.9, 38.7 / 38.7, 33.2 / 33.3, 70.4 / 70.0, 89.2 / 89.0.
 // grid_enter: one thread, after pdl_wait() (the control words may be the predecessor's until then); returns how many CTAs
 // began before this one.
 __device__ __forceinline__ unsigned grid_enter(WsCtrl *ctrl) {
