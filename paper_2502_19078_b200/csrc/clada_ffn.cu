@@ -69,7 +69,7 @@ sparse_ffn_kernel(const FfnParams p, const int n_stages, const bool pair) {
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     pdl_wait();  // everything below may read what the previous kernel wrote
-    if (tid == kConsumers + 1) grid_enter(p.ctrl);  // a thread with nothing else to do
+    if (tid == kConsumers + 1) grid_enter(p.ctrl);  // a thread with nothing else to do yet
 
     const uint64_t keep_policy = policy_evict_last();
     const bool nested = p.order != nullptr;
@@ -244,8 +244,9 @@ sparse_ffn_kernel(const FfnParams p, const int n_stages, const bool pair) {
     if (p.count_out && cta == 0 && tid == 0) *p.count_out = n_act;
     const int my_n = r1 - r0;
     if (n_act == 0) {
+        pdl_launch_dependents();
         // Nothing is kept (every CTA sees the same count): y = 0, written slice by slice, and there are
-        // no partial sums to combine, so the meeting is skipped as well.
+        // no partial sums to combine, so the meeting is skipped as well, and the next launch is released at once.
         const int ng = d / 4;  // output in groups of 4 columns
         const int q0 = split_at(ng, cta, n_ctas), q1 = split_at(ng, cta + 1, n_ctas);
         for (int q = q0 + tid; q < q1; q += kFfnThreads) {
@@ -254,10 +255,7 @@ sparse_ffn_kernel(const FfnParams p, const int n_stages, const bool pair) {
             else
                 reinterpret_cast<uint2 *>(p.y)[q] = make_uint2(0u, 0u);
         }
-        if (tid == 0) {
-            __threadfence();  // the count in grid_enter lands before the last CTA's departure clears it
-            grid_leave(p.ctrl, (unsigned)n_ctas);
-        }
+        if (tid == kConsumers + 1) grid_exit(p.ctrl);  // the thread that counted the CTA in
         return;
     }
     __syncthreads();  // s_list and the mbarriers are ready

@@ -28,6 +28,12 @@ constexpr unsigned kBarrierSpinLimit = 1u << 22;  // polls of an L2 word: gives 
 __device__ __forceinline__ unsigned grid_enter(WsCtrl *ctrl) {
     return (unsigned)(atomicAdd(reinterpret_cast<unsigned long long *>(ctrl), 1ull << 32) >> 32);
 }
+// grid_exit: instead of a meeting that no CTA of the launch comes to, by the thread that called grid_enter.  It takes its
+// count back, so nothing has to be ordered or cleared (launches of 4096 x 11008 that keep nothing, in a graph: 4.7 us with a
+// departure and its reset, 3.9 this way).
+__device__ __forceinline__ void grid_exit(WsCtrl *ctrl) {
+    atomicAdd(reinterpret_cast<unsigned long long *>(ctrl), 0ull - (1ull << 32));
+}
 // grid_leave: one thread of every CTA, once the CTA has nothing more to read from the control words; between it and
 // grid_enter lies a device-wide fence (grid_meet has one), or a late count could land after the last CTA's reset.
 __device__ __forceinline__ void grid_leave(WsCtrl *ctrl, unsigned n_ctas) {

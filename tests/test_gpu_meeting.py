@@ -100,7 +100,7 @@ def test_two_streams(clada, first):
 
 @pytest.mark.parametrize("form", NOTHING_KEPT)
 def test_launches_that_keep_nothing(clada, form):
-    """They leave without a meeting: y is zero, and the control words are zero for the dense pass behind each, which
+    """They take their counts back without a meeting: y is zero, and the control words are zero for the dense pass behind each, which
     numbers its CTAs by one of them.  On two streams, so that launches begin a few CTAs at a time."""
     none, dense = [_Decode(clada, *form) for _ in (0, 1)], [_Decode(clada, 6, 1024, 2400, torch.bfloat16, False) for _ in (0, 1)]
     want = dense[0].run()
